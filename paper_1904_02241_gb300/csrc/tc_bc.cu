@@ -19,8 +19,8 @@
 //   dep[v] = sum over out-neighbours w of depth L+1 of sigma[v] / sigma[w] * (1 + dep[w])
 //          = sigma[v] * sum over those w of coef[w],   coef[w] = (1 + dep[w]) / sigma[w],
 // so each vertex divides once (when its dependency is known) and each edge only adds; FP64
-// division is slow on this GPU.  One warp per vertex: each lane adds its strided share of the
-// row in order, then a fixed shuffle tree adds the lane sums; every vertex other than the source
+// division is slow on this GPU.  A lane group, a warp or a CTA per vertex: each lane adds its strided
+// share of the row in order, then a fixed tree adds the lane sums; every vertex other than the source
 // adds dep[v] to its score.  Operations are rounded one by one (no fused multiply-add).  A
 // vertex's dependency reads only final values of the next level, so the order of a level's list
 // (which the forward sweep fills as vertices are reached) does not change any result.
@@ -50,14 +50,6 @@ __global__ void k_bc_zero(int32_t V, double *score) {
         score[v] = 0.0;
 }
 
-// A vertex x joins level L+1: it is appended to the next frontier and its out-degree is added to
-// the next frontier's out-edge count (the direction rule's m_f).
-__device__ __forceinline__ void bc_reach(int32_t x, const int32_t *__restrict__ out_rowptr, int32_t *next,
-                                         unsigned *next_count, unsigned long long *next_deg) {
-    next[atomicAdd(next_count, 1u)] = x;
-    atomicAdd(next_deg, (unsigned long long)(__ldg(out_rowptr + x + 1) - __ldg(out_rowptr + x)));
-}
-
 // out-degree of every frontier vertex (for the push level's edge prefix)
 __global__ void k_bc_front_deg(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ front, int64_t nf,
                                int32_t *deg) {
@@ -71,91 +63,116 @@ __global__ void k_bc_front_deg(const int32_t *__restrict__ rowptr, const int32_t
 // concatenated out-rows (pre = exclusive prefix of their lengths, total = the sum) and finds its
 // row by binary search, so a hub's row spreads over the whole grid.  The first edge to reach w
 // claims it with a CAS on depth; every edge into a vertex of depth L+1 adds sigma[u] (integers
-// below 2^53: exact in any order).
+// below 2^53: exact in any order).  The next frontier and its out-edge count (the direction rule's
+// m_f) go through the warps' queues.
 __global__ void __launch_bounds__(BC_THREADS) k_bc_push_edges(const int32_t *__restrict__ rowptr,
                                                               const int32_t *__restrict__ colidx,
                                                               const int32_t *__restrict__ front, int64_t nf,
                                                               const int64_t *__restrict__ pre, int64_t total,
                                                               int32_t L, int32_t *depth, double *sigma, int32_t *next,
-                                                              unsigned *next_count, unsigned long long *next_deg) {
+                                                              unsigned long long *count) {
+    __shared__ int32_t wq_buf[BC_WARPS * WQ_ENTRIES];
+    WarpQueue wq(wq_buf);
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += stride) {
-        int64_t lo = 0, hi = nf;  // last i with pre[i] <= e
-        while (hi - lo > 1) {
-            const int64_t mid = (lo + hi) >> 1;
-            if (__ldg(pre + mid) <= e) lo = mid; else hi = mid;
-        }
-        const int32_t u = __ldg(front + lo);
-        const int32_t w = __ldg(colidx + __ldg(rowptr + u) + (e - __ldg(pre + lo)));
-        int32_t dw = *(volatile int32_t *)(depth + w);
-        if (dw == -1) {
-            dw = atomicCAS(depth + w, -1, L + 1);
-            if (dw == -1) {  // this edge reached w first
-                dw = L + 1;
-                bc_reach(w, rowptr, next, next_count, next_deg);
+    // warp-uniform loop: the queue's ballots see the whole warp
+    for (int64_t base = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); base < total; base += stride) {
+        const int64_t e = base + (threadIdx.x & 31);
+        bool claimed = false;
+        int32_t w = 0, deg = 0;
+        if (e < total) {
+            int64_t lo = 0, hi = nf;  // last i with pre[i] <= e
+            while (hi - lo > 1) {
+                const int64_t mid = (lo + hi) >> 1;
+                if (__ldg(pre + mid) <= e) lo = mid; else hi = mid;
             }
+            const int32_t u = __ldg(front + lo);
+            w = __ldg(colidx + __ldg(rowptr + u) + (e - __ldg(pre + lo)));
+            int32_t dw = *(volatile int32_t *)(depth + w);
+            if (dw == -1) {
+                dw = atomicCAS(depth + w, -1, L + 1);
+                if (dw == -1) {  // this edge reached w first
+                    dw = L + 1;
+                    claimed = true;
+                    deg = __ldg(rowptr + w + 1) - __ldg(rowptr + w);
+                }
+            }
+            if (dw == L + 1) atomicAdd(sigma + w, sigma[u]);
         }
-        if (dw == L + 1) atomicAdd(sigma + w, sigma[u]);
+        wq.push(claimed, w, deg, next, count);
     }
+    wq.finish(next, count, count + 1);
 }
 
-// pull level L, short in-rows: a thread per unreached vertex
+// pull level L.  The first nhubs CTAs take a hub row each (more than hub_degree in-edges); in the
+// others a warp takes 32 consecutive vertices: a lane sums a short in-row of an unreached one, the
+// warp the rows of BC_LONG or more in-edges.  The sums are integers: exact in any order.  One
+// launch instead of one per class: rows of the classes share the reads of depth and the row
+// offsets, and hubs spread over a CTA instead of one warp.
 __global__ void __launch_bounds__(BC_THREADS) k_bc_pull(const int32_t *__restrict__ in_rowptr,
                                                         const int32_t *__restrict__ in_colidx,
-                                                        const int32_t *__restrict__ out_rowptr, int32_t V, int32_t L,
-                                                        int32_t *depth, double *sigma, int32_t *next,
-                                                        unsigned *next_count, unsigned long long *next_deg) {
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < V; v += (int64_t)gridDim.x * blockDim.x) {
-        if (depth[v] != -1) continue;
-        const int32_t s = in_rowptr[v], e = in_rowptr[v + 1];
-        if (e - s >= BC_LONG) continue;  // k_bc_pull_long
+                                                        const int32_t *__restrict__ out_rowptr, int32_t V,
+                                                        const int32_t *__restrict__ hubs, int32_t nhubs,
+                                                        int32_t hub_degree, int32_t L, int32_t *depth, double *sigma,
+                                                        int32_t *next, unsigned long long *count) {
+    __shared__ int32_t wq_buf[BC_WARPS * WQ_ENTRIES];
+    __shared__ double red[32];
+    WarpQueue wq(wq_buf);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if ((int32_t)blockIdx.x < nhubs) {
+        const int32_t v = hubs[blockIdx.x];
+        const bool open = depth[v] == -1;  // the same for the whole CTA: only this CTA sets it
         double acc = 0.0;
-        bool hit = false;
-        for (int32_t i = s; i < e; ++i) {
-            const int32_t u = in_colidx[i];
-            if (depth[u] == L) {
-                acc = __dadd_rn(acc, sigma[u]);
-                hit = true;
+        if (open)
+            for (int32_t i = in_rowptr[v] + threadIdx.x; i < in_rowptr[v + 1]; i += BC_THREADS) {
+                const int32_t u = in_colidx[i];
+                if (depth[u] == L) acc = __dadd_rn(acc, sigma[u]);
             }
-        }
+        acc = block_sum<double>(acc, red);  // every thread has read depth[v] by now
+        const bool hit = open && acc != 0.0 && threadIdx.x == 0;  // sigma of a reached vertex is at least 1
         if (hit) {
             depth[v] = L + 1;
             sigma[v] = acc;
-            bc_reach((int32_t)v, out_rowptr, next, next_count, next_deg);
         }
-    }
-}
-
-// pull level L, long in-rows: a warp per unreached vertex of the long-row list
-__global__ void __launch_bounds__(BC_THREADS) k_bc_pull_long(const int32_t *__restrict__ in_rowptr,
-                                                             const int32_t *__restrict__ in_colidx,
-                                                             const int32_t *__restrict__ out_rowptr,
-                                                             const int32_t *__restrict__ longrows, int32_t nlong,
-                                                             int32_t L, int32_t *depth, double *sigma, int32_t *next,
-                                                             unsigned *next_count, unsigned long long *next_deg) {
-    const int lane = threadIdx.x & 31;
-    const int64_t nw = (int64_t)gridDim.x * BC_WARPS;
-    for (int64_t k = (blockIdx.x * (int64_t)BC_THREADS + threadIdx.x) >> 5; k < nlong; k += nw) {
-        const int32_t v = longrows[k];
-        if (depth[v] != -1) continue;  // the same value for the whole warp
-        double acc = 0.0;
-        bool hit = false;
-        for (int32_t i = in_rowptr[v] + lane; i < in_rowptr[v + 1]; i += 32) {
-            const int32_t u = in_colidx[i];
-            if (depth[u] == L) {
-                acc = __dadd_rn(acc, sigma[u]);
-                hit = true;
+        wq.push(hit, v, hit ? out_rowptr[v + 1] - out_rowptr[v] : 0, next, count);
+    } else {
+        const int64_t nw = (int64_t)(gridDim.x - nhubs) * BC_WARPS;
+        for (int64_t grp = (int64_t)(blockIdx.x - nhubs) * BC_WARPS + warp; grp * 32 < V; grp += nw) {
+            const int64_t v = grp * 32 + lane;
+            int32_t s = 0, e = 0;
+            if (v < V && depth[v] == -1) {
+                s = in_rowptr[v];
+                e = in_rowptr[v + 1];
+                if (e - s > hub_degree) e = s;  // its own CTA
             }
-        }
+            double acc = 0.0;
+            if (e - s < BC_LONG)
+                for (int32_t i = s; i < e; ++i) {
+                    const int32_t u = in_colidx[i];
+                    if (depth[u] == L) acc = __dadd_rn(acc, sigma[u]);
+                }
+            unsigned long_rows = __ballot_sync(0xffffffffu, e - s >= BC_LONG);
+            while (long_rows) {
+                const int l = __ffs(long_rows) - 1;
+                long_rows &= long_rows - 1;
+                const int32_t ls = __shfl_sync(0xffffffffu, s, l), le = __shfl_sync(0xffffffffu, e, l);
+                double w = 0.0;
+                for (int32_t i = ls + lane; i < le; i += 32) {
+                    const int32_t u = in_colidx[i];
+                    if (depth[u] == L) w = __dadd_rn(w, sigma[u]);
+                }
 #pragma unroll
-        for (int d = 16; d > 0; d >>= 1) acc = __dadd_rn(acc, __shfl_xor_sync(0xffffffffu, acc, d));
-        hit = __any_sync(0xffffffffu, hit);
-        if (hit && lane == 0) {
-            depth[v] = L + 1;
-            sigma[v] = acc;
-            bc_reach(v, out_rowptr, next, next_count, next_deg);
+                for (int d = 16; d > 0; d >>= 1) w = __dadd_rn(w, __shfl_xor_sync(0xffffffffu, w, d));
+                if (lane == l) acc = w;
+            }
+            const bool hit = acc != 0.0;
+            if (hit) {
+                depth[v] = L + 1;
+                sigma[v] = acc;
+            }
+            wq.push(hit, (int32_t)v, hit ? __ldg(out_rowptr + v + 1) - __ldg(out_rowptr + v) : 0, next, count);
         }
     }
+    wq.finish(next, count, count + 1);
 }
 
 // Blocked pull level (TOCAB, Sec. 3.3 with sigma sums as the "next" values): local row r of a
@@ -210,8 +227,10 @@ __global__ void __launch_bounds__(BC_THREADS) k_bc_block_merge(const double *__r
                                                                int32_t nranges, int32_t k, int32_t V, int32_t L,
                                                                const int32_t *__restrict__ out_rowptr,
                                                                int32_t *depth, double *sigma, int32_t *next,
-                                                               unsigned *next_count, unsigned long long *next_deg) {
+                                                               unsigned long long *count) {
     extern __shared__ double bacc[];  // [k]
+    __shared__ int32_t wq_buf[BC_WARPS * WQ_ENTRIES];
+    WarpQueue wq(wq_buf);
     for (int32_t j = blockIdx.x; j < nranges; j += gridDim.x) {
         const int32_t vbase = j * k;
         for (int32_t t = threadIdx.x; t < k; t += BC_THREADS) bacc[t] = 0.0;
@@ -225,17 +244,21 @@ __global__ void __launch_bounds__(BC_THREADS) k_bc_block_merge(const double *__r
             }
             __syncthreads();
         }
-        for (int32_t t = threadIdx.x; t < k && vbase + t < V; t += BC_THREADS) {
-            const double x = bacc[t];
+        for (int32_t t0 = 0; t0 < k && vbase + t0 < V; t0 += BC_THREADS) {  // the same steps for the whole CTA
+            const int32_t t = t0 + (int32_t)threadIdx.x;
             const int32_t v = vbase + t;
-            if (x != 0.0 && depth[v] == -1) {
+            const bool in = t < k && v < V;
+            const double x = in ? bacc[t] : 0.0;
+            const bool hit = x != 0.0 && depth[v] == -1;
+            if (hit) {
                 depth[v] = L + 1;
                 sigma[v] = x;
-                bc_reach(v, out_rowptr, next, next_count, next_deg);
             }
+            wq.push(hit, v, hit ? __ldg(out_rowptr + v + 1) - __ldg(out_rowptr + v) : 0, next, count);
         }
         __syncthreads();
     }
+    wq.finish(next, count, count + 1);
 }
 
 // dependency of v from t = the sum over its children of (1 + dep[w]) / sigma[w]: dep[v] =
@@ -249,86 +272,71 @@ __device__ __forceinline__ void bc_dep_update(int32_t v, double t, int32_t sourc
 }
 
 // Dependencies of the vertices of depth L (those of depth L+1 are final), by out-degree class:
-// up to BC_SMALL a group of 8 lanes (four vertices per warp), up to the hub degree a warp, above
-// it a CTA (k_bc_backward_hub).  Each class adds in a fixed order, so scores repeat bit for bit.
+// above the hub degree a CTA each (the first nhubs CTAs, one per hub of the graph's list; hubs at
+// other depths leave at once), up to BC_SMALL a group of 8 lanes (four vertices per warp), between
+// them the warp that met the vertex.  Each class adds in a fixed order, so scores repeat bit for bit.
+// One launch per level instead of one per class, which read the level's list twice and cost three
+// launches on the small levels (4 sources on a symmetrised R-MAT 18: 1,077 us of 2,096 in 75 launches).
 constexpr int32_t BC_SMALL = 64;
 
-__global__ void __launch_bounds__(BC_THREADS) k_bc_backward_small(const int32_t *__restrict__ rowptr,
-                                                                  const int32_t *__restrict__ colidx,
-                                                                  const int32_t *__restrict__ level_list, int64_t n,
-                                                                  int32_t L, int32_t source, int32_t small_max,
-                                                                  const int32_t *__restrict__ depth,
-                                                                  const double *__restrict__ sigma, double *coef,
-                                                                  double *score) {
+__global__ void __launch_bounds__(BC_THREADS) k_bc_backward(const int32_t *__restrict__ rowptr,
+                                                            const int32_t *__restrict__ colidx,
+                                                            const int32_t *__restrict__ level_list, int64_t n,
+                                                            const int32_t *__restrict__ hubs, int32_t nhubs, int32_t L,
+                                                            int32_t source, int32_t small_max, int32_t hub_degree,
+                                                            const int32_t *__restrict__ depth,
+                                                            const double *__restrict__ sigma, double *coef,
+                                                            double *score) {
+    __shared__ double red[32];
+    if ((int32_t)blockIdx.x < nhubs) {
+        const int32_t v = hubs[blockIdx.x];
+        if (depth[v] != L) return;  // the same for the whole CTA
+        double t = 0.0;
+        for (int32_t e = rowptr[v] + threadIdx.x; e < rowptr[v + 1]; e += BC_THREADS) {
+            const int32_t w = colidx[e];
+            if (depth[w] == L + 1) t = __dadd_rn(t, coef[w]);
+        }
+        t = block_sum<double>(t, red);
+        if (threadIdx.x == 0) bc_dep_update(v, t, source, sigma, coef, score);
+        return;
+    }
     const int lane = threadIdx.x & 31, sub = lane & 7;
-    const int64_t step = (int64_t)gridDim.x * BC_WARPS * 4;
+    const int64_t step = (int64_t)(gridDim.x - nhubs) * BC_WARPS * 4;
     // warp-uniform loop: the shuffles below see the whole warp
-    for (int64_t base = ((blockIdx.x * (int64_t)BC_THREADS + threadIdx.x) >> 5) * 4; base < n; base += step) {
+    for (int64_t base = (((int64_t)(blockIdx.x - nhubs) * BC_THREADS + threadIdx.x) >> 5) * 4; base < n; base += step) {
         const int64_t k = base + (lane >> 3);
         int32_t v = -1, s = 0, e = 0;
         if (k < n) {
             v = level_list[k];
             s = rowptr[v];
             e = rowptr[v + 1];
-            if (e - s > small_max) {  // a larger class
-                v = -1;
-                e = s;
-            }
         }
+        const bool small = e - s <= small_max;
         double t = 0.0;
-        for (int32_t i = s + sub; i < e; i += 8) {
-            const int32_t w = colidx[i];
-            if (depth[w] == L + 1) t = __dadd_rn(t, coef[w]);
-        }
+        if (small)
+            for (int32_t i = s + sub; i < e; i += 8) {
+                const int32_t w = colidx[i];
+                if (depth[w] == L + 1) t = __dadd_rn(t, coef[w]);
+            }
 #pragma unroll
         for (int q = 4; q > 0; q >>= 1) t = __dadd_rn(t, __shfl_xor_sync(0xffffffffu, t, q));
-        if (sub == 0 && v >= 0) bc_dep_update(v, t, source, sigma, coef, score);
-    }
-}
-
-__global__ void __launch_bounds__(BC_THREADS) k_bc_backward(const int32_t *__restrict__ rowptr,
-                                                            const int32_t *__restrict__ colidx,
-                                                            const int32_t *__restrict__ level_list, int64_t n,
-                                                            int32_t L, int32_t source, int32_t small_max,
-                                                            int32_t hub_degree, const int32_t *__restrict__ depth,
-                                                            const double *__restrict__ sigma, double *coef,
-                                                            double *score) {
-    const int lane = threadIdx.x & 31;
-    const int64_t nw = (int64_t)gridDim.x * BC_WARPS;
-    for (int64_t k = (blockIdx.x * (int64_t)BC_THREADS + threadIdx.x) >> 5; k < n; k += nw) {
-        const int32_t v = level_list[k];
-        const int32_t deg = rowptr[v + 1] - rowptr[v];
-        if (deg <= small_max || deg > hub_degree) continue;  // the same for the whole warp
-        double t = 0.0;  // sum of (1 + dep[w]) / sigma[w] over the children w
-        for (int32_t e = rowptr[v] + lane; e < rowptr[v + 1]; e += 32) {
-            const int32_t w = colidx[e];
-            if (depth[w] == L + 1) t = __dadd_rn(t, coef[w]);
-        }
+        if (sub == 0 && v >= 0 && small) bc_dep_update(v, t, source, sigma, coef, score);
+        unsigned wm = __ballot_sync(0xffffffffu, sub == 0 && !small && e - s <= hub_degree);
+        while (wm) {
+            const int l = __ffs(wm) - 1;
+            wm &= wm - 1;
+            const int32_t lv = __shfl_sync(0xffffffffu, v, l);
+            const int32_t ls = __shfl_sync(0xffffffffu, s, l), le = __shfl_sync(0xffffffffu, e, l);
+            double x = 0.0;
+            for (int32_t i = ls + lane; i < le; i += 32) {
+                const int32_t w = colidx[i];
+                if (depth[w] == L + 1) x = __dadd_rn(x, coef[w]);
+            }
 #pragma unroll
-        for (int q = 16; q > 0; q >>= 1) t = __dadd_rn(t, __shfl_xor_sync(0xffffffffu, t, q));
-        if (lane == 0) bc_dep_update(v, t, source, sigma, coef, score);
+            for (int q = 16; q > 0; q >>= 1) x = __dadd_rn(x, __shfl_xor_sync(0xffffffffu, x, q));
+            if (lane == 0) bc_dep_update(lv, x, source, sigma, coef, score);
+        }
     }
-}
-
-// the hubs of depth L: a CTA per hub of the graph's hub list, threads striding the out-row and a
-// fixed-order block reduction (deterministic for the fixed launch shape); hubs at other depths
-// leave at once
-__global__ void __launch_bounds__(BC_THREADS) k_bc_backward_hub(const int32_t *__restrict__ rowptr,
-                                                                const int32_t *__restrict__ colidx,
-                                                                const int32_t *__restrict__ hubs, int32_t L,
-                                                                int32_t source, const int32_t *__restrict__ depth,
-                                                                const double *__restrict__ sigma, double *coef,
-                                                                double *score) {
-    __shared__ double red[32];
-    const int32_t v = hubs[blockIdx.x];
-    if (depth[v] != L) return;  // the same for the whole CTA
-    double t = 0.0;
-    for (int32_t e = rowptr[v] + threadIdx.x; e < rowptr[v + 1]; e += BC_THREADS) {
-        const int32_t w = colidx[e];
-        if (depth[w] == L + 1) t = __dadd_rn(t, coef[w]);
-    }
-    t = block_sum<double>(t, red);
-    if (threadIdx.x == 0) bc_dep_update(v, t, source, sigma, coef, score);
 }
 
 // A level runs in the push direction while its frontier's out-edges are fewer than
@@ -337,9 +345,8 @@ __global__ void __launch_bounds__(BC_THREADS) k_bc_backward_hub(const int32_t *_
 constexpr int64_t BC_PUSH_RATIO = 14;
 
 struct BcScratch {
-    DevBuf depth, sigma, coef, score, order, counter, longrows, bpartial;
+    DevBuf depth, sigma, coef, score, order, counter, bpartial;
     DevBuf fdeg, fpre, fws;  // push levels: frontier out-degrees, their prefix, scan scratch
-    int32_t nlong = 0;
     std::vector<int64_t> off;  // level L of `order` is [off[L], off[L+1])
     int grid = 1;
     int setup(const tc_graph *g, bool need_score, cudaStream_t s, const tc_part *part = nullptr) {
@@ -361,7 +368,6 @@ struct BcScratch {
         TC_TRY(fdeg.alloc((size_t)V * 4 + 16));
         TC_TRY(fpre.alloc((size_t)V * 8 + 16));
         TC_TRY(fws.alloc((size_t)(scan_ws_elems(V) + 16) * 8));
-        TC_TRY(collect_hubs(g->in_rowptr.as<int32_t>(), V, BC_LONG - 1, &longrows, &nlong, s));
         return TC_OK;
     }
 };
@@ -373,8 +379,7 @@ static int bc_forward_impl(const tc_graph *g, const tc_part *part, int32_t sourc
     const int32_t V = g->V;
     int32_t *depth = w.depth.as<int32_t>(), *order = w.order.as<int32_t>();
     double *sigma = w.sigma.as<double>();
-    unsigned *cnt = w.counter.as<unsigned>();
-    unsigned long long *ndeg = reinterpret_cast<unsigned long long *>(w.counter.as<char>() + 8);
+    unsigned long long *cnt = w.counter.as<unsigned long long>();  // found vertices, their out-edges
     const int32_t *orp = g->out_rowptr.as<int32_t>();
     k_bc_init<<<w.grid, BC_THREADS, 0, s>>>(V, source, depth, sigma, w.coef.as<double>(), order);
     TC_LAUNCH_CHECK();
@@ -399,8 +404,7 @@ static int bc_forward_impl(const tc_graph *g, const tc_part *part, int32_t sourc
                 const int64_t want = (m_f + BC_THREADS - 1) / BC_THREADS;
                 const int grid = (int)(want < w.grid ? want : w.grid);
                 k_bc_push_edges<<<grid, BC_THREADS, 0, s>>>(orp, g->out_colidx.as<int32_t>(), order + f0, nf,
-                                                            w.fpre.as<int64_t>(), m_f, L, depth, sigma, next, cnt,
-                                                            ndeg);
+                                                            w.fpre.as<int64_t>(), m_f, L, depth, sigma, next, cnt);
                 TC_LAUNCH_CHECK();
             }
             ++np;
@@ -415,23 +419,18 @@ static int bc_forward_impl(const tc_graph *g, const tc_part *part, int32_t sourc
             const int mgrid = part->nranges < w.grid ? (part->nranges > 0 ? part->nranges : 1) : w.grid;
             k_bc_block_merge<<<mgrid, BC_THREADS, smem, s>>>(w.bpartial.as<double>(), part->id_map.as<int32_t>(),
                                                              part->merge_off.as<int32_t>(), part->B, part->nranges,
-                                                             part->k, V, L, orp, depth, sigma, next, cnt, ndeg);
+                                                             part->k, V, L, orp, depth, sigma, next, cnt);
             TC_LAUNCH_CHECK();
         } else {
-            k_bc_pull<<<w.grid, BC_THREADS, 0, s>>>(g->in_rowptr.as<int32_t>(), g->in_colidx.as<int32_t>(), orp, V,
-                                                    L, depth, sigma, next, cnt, ndeg);
+            k_bc_pull<<<w.grid + g->num_in_hubs, BC_THREADS, 0, s>>>(
+                g->in_rowptr.as<int32_t>(), g->in_colidx.as<int32_t>(), orp, V, g->in_hubs.as<int32_t>(),
+                g->num_in_hubs, g->hub_degree, L, depth, sigma, next, cnt);
             TC_LAUNCH_CHECK();
-            if (w.nlong > 0) {
-                k_bc_pull_long<<<w.grid, BC_THREADS, 0, s>>>(g->in_rowptr.as<int32_t>(), g->in_colidx.as<int32_t>(),
-                                                             orp, w.longrows.as<int32_t>(), w.nlong, L, depth, sigma,
-                                                             next, cnt, ndeg);
-                TC_LAUNCH_CHECK();
-            }
         }
-        unsigned long long hc[2] = {0, 0};  // found (low word of the first), out-edges of the found
+        unsigned long long hc[2] = {0, 0};
         TC_CUDA(cudaMemcpyAsync(hc, cnt, 16, cudaMemcpyDeviceToHost, s));
         TC_CUDA(cudaStreamSynchronize(s));
-        const unsigned found = (unsigned)(hc[0] & 0xFFFFFFFFull);
+        const unsigned long long found = hc[0];
         if (found == 0) break;
         w.off.push_back(reached + (int64_t)found);
         m_f = (int64_t)hc[1];
@@ -512,25 +511,11 @@ static int bc_impl(const tc_graph *g, const tc_part *part, const int32_t *source
             const int64_t a = w.off[(size_t)L], n = w.off[(size_t)L + 1] - a;
             const int64_t want4 = (n + 4 * BC_WARPS - 1) / (4 * BC_WARPS);
             const int grid4 = (int)(want4 < w.grid ? (want4 > 0 ? want4 : 1) : w.grid);
-            k_bc_backward_small<<<grid4, BC_THREADS, 0, s>>>(g->out_rowptr.as<int32_t>(), g->out_colidx.as<int32_t>(),
-                                                             w.order.as<int32_t>() + a, n, L, sources[k], small_max,
-                                                             w.depth.as<int32_t>(), w.sigma.as<double>(),
-                                                             w.coef.as<double>(), score);
+            k_bc_backward<<<grid4 + g->num_out_hubs, BC_THREADS, 0, s>>>(
+                g->out_rowptr.as<int32_t>(), g->out_colidx.as<int32_t>(), w.order.as<int32_t>() + a, n,
+                g->out_hubs.as<int32_t>(), g->num_out_hubs, L, sources[k], small_max, g->hub_degree,
+                w.depth.as<int32_t>(), w.sigma.as<double>(), w.coef.as<double>(), score);
             TC_LAUNCH_CHECK();
-            const int64_t want = (n + BC_WARPS - 1) / BC_WARPS;
-            const int grid = (int)(want < w.grid ? (want > 0 ? want : 1) : w.grid);
-            k_bc_backward<<<grid, BC_THREADS, 0, s>>>(g->out_rowptr.as<int32_t>(), g->out_colidx.as<int32_t>(),
-                                                      w.order.as<int32_t>() + a, n, L, sources[k], small_max,
-                                                      g->hub_degree,
-                                                      w.depth.as<int32_t>(), w.sigma.as<double>(),
-                                                      w.coef.as<double>(), score);
-            TC_LAUNCH_CHECK();
-            if (g->num_out_hubs > 0) {
-                k_bc_backward_hub<<<g->num_out_hubs, BC_THREADS, 0, s>>>(
-                    g->out_rowptr.as<int32_t>(), g->out_colidx.as<int32_t>(), g->out_hubs.as<int32_t>(), L,
-                    sources[k], w.depth.as<int32_t>(), w.sigma.as<double>(), w.coef.as<double>(), score);
-                TC_LAUNCH_CHECK();
-            }
         }
     }
     if (!dev_out) TC_CUDA(cudaMemcpyAsync(scores_out, score, (size_t)V * 8, cudaMemcpyDeviceToHost, s));

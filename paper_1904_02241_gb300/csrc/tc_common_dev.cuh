@@ -177,4 +177,60 @@ __device__ __forceinline__ bool grid_sum2_last_cta(double a, double b, double *p
     return true;
 }
 
+// Appends to a queue in global memory, staged per warp in shared memory: `count` moves by one atomic
+// per 32 entries (and one per CTA at the end) instead of one per entry or per warp step.  An atomic
+// per entry on one address bounded the traversal levels that had it (BC from 4 sources on a
+// symmetrised R-MAT 18, with the classes of a level in one launch: 2,552 to 1,698 us).  The entries' weights (out-degrees) are summed
+// per lane and leave as one atomic per CTA.  All threads of the CTA call finish() once.
+constexpr int WQ_ENTRIES = 64;  // per warp: below 32 entries wait, at most 32 arrive at once
+struct WarpQueue {
+    int32_t *buf;                // this warp's WQ_ENTRIES words of shared memory
+    int32_t n = 0;               // entries waiting (warp-uniform)
+    unsigned long long w = 0;    // this lane's weights
+    __device__ explicit WarpQueue(int32_t *smem) : buf(smem + (threadIdx.x >> 5) * WQ_ENTRIES) {}
+    // The whole warp calls it; lanes with `has` append v.
+    __device__ __forceinline__ void push(bool has, int32_t v, int32_t weight, int32_t *queue, unsigned long long *count) {
+        const int lane = threadIdx.x & 31;
+        const unsigned m = __ballot_sync(0xffffffffu, has);
+        if (m == 0u) return;
+        if (has) {
+            buf[n + __popc(m & ((1u << lane) - 1u))] = v;
+            w += (unsigned long long)weight;
+        }
+        n += __popc(m);
+        if (n < 32) return;
+        __syncwarp();
+        unsigned long long base = 0;
+        if (lane == 0) base = atomicAdd(count, 32ull);
+        base = __shfl_sync(0xffffffffu, base, 0);
+        queue[base + lane] = buf[lane];
+        const int32_t rest = lane < n - 32 ? buf[32 + lane] : 0;
+        __syncwarp();
+        if (lane < n - 32) buf[lane] = rest;
+        n -= 32;
+        __syncwarp();
+    }
+    // The waiting entries of all warps, and the CTA's weights (added to *weight_sum).
+    __device__ __forceinline__ void finish(int32_t *queue, unsigned long long *count, unsigned long long *weight_sum) {
+        __shared__ int32_t wq_n[32];
+        __shared__ unsigned long long wq_red[32], wq_base;
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
+        const unsigned long long sum = block_sum<unsigned long long>(w, wq_red);
+        if (lane == 0) wq_n[warp] = n;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            int32_t t = 0;
+            for (int i = 0; i < nw; ++i) {
+                const int32_t x = wq_n[i];
+                wq_n[i] = t;
+                t += x;
+            }
+            wq_base = t > 0 ? atomicAdd(count, (unsigned long long)t) : 0ull;
+            if (sum) atomicAdd(weight_sum, sum);
+        }
+        __syncthreads();
+        if (lane < n) queue[wq_base + wq_n[warp] + lane] = buf[lane];
+    }
+};
+
 }  // namespace tc

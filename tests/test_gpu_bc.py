@@ -158,3 +158,18 @@ def test_blocked_bc_refuses_other_partitions(T):
         T.bc(G, [0], part=T.tocab_partition(G, T.TC_PUSH, 2))
     with pytest.raises(T.TocabError):
         T.bc(G, [0], part=T.tocab_partition(G, T.TC_PULL, 2, order="outdegree"))
+
+
+@pytest.mark.parametrize("n", [31, 32, 33, 63, 64, 65, 255, 256, 257, 3000])
+def test_levels_around_the_warp_queues_flush_sizes(T, n):
+    """A level of n vertices through the warps' append queues (flushed 32 at a time): a star pushes n
+    leaves from its hub, and from a leaf pulls or pushes n - 1; every score exact."""
+    g = gg.star(n)
+    rp, ci = g.numpy()
+    G = _load(T, g)
+    for s in (0, 1):
+        d, sg = T.bc_forward(G, s)
+        wd, ws = oracle.bc_forward(g.V, rp, ci, s)
+        assert np.array_equal(d.cpu().numpy(), wd) and np.array_equal(sg.cpu().numpy(), ws)
+    got = T.bc(G, [0, 1]).cpu().numpy()
+    np.testing.assert_allclose(got, oracle.bc(g.V, rp, ci, [0, 1]), rtol=1e-12, atol=0)
