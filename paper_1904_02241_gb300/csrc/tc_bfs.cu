@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(BFS_THREADS) k_bfs_merge(const uint32_t *__res
 // Push (top-down, data-driven) levels for small frontiers (Sec. 3.3: the push phases of the
 // push-pull-push schedule, Alg. 3 without sigma): every frontier vertex in the queue scans its
 // out-edges; an unvisited neighbour is claimed with an atomic OR on the visited bitmap, gets
-// its level, joins the next bitmap and is appended to the next queue (warp-aggregated).
+// its level, joins the next bitmap and is appended to the next queue (through its warp's queue).
 // Edge-balanced push level: the out-degrees of the queue are scanned (pre[q+1]); thread t takes
 // edges t, t + stride, ... of the frontier's concatenated out-rows, finds its row by binary
 // search in pre, and claims the neighbour as above.  Hubs spread over the whole grid.
@@ -216,6 +216,8 @@ __global__ void __launch_bounds__(BFS_THREADS) k_bfs_push_edges(const int32_t *_
                                                                 uint32_t *visited, uint32_t *next, int32_t *level,
                                                                 int32_t new_level, int32_t *next_queue,
                                                                 unsigned long long *count) {
+    __shared__ int32_t wq_buf[BFS_WARPS * WQ_ENTRIES];
+    WarpQueue wq(wq_buf);
     const int lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < total; base += stride) {
@@ -236,23 +238,15 @@ __global__ void __launch_bounds__(BFS_THREADS) k_bfs_push_edges(const int32_t *_
                 claimed = !(old & bit);
             }
         }
-        const unsigned cm = __ballot_sync(0xffffffffu, claimed);
-        if (cm) {
-            int32_t pos0 = 0;
-            if (lane == __ffs(cm) - 1) pos0 = (int32_t)atomicAdd(count, (unsigned long long)__popc(cm));
-            pos0 = __shfl_sync(0xffffffffu, pos0, __ffs(cm) - 1);
-            unsigned long long dg = 0;
-            if (claimed) {
-                level[v] = new_level;
-                atomicOr(next + (v >> 5), 1u << (v & 31));
-                next_queue[pos0 + __popc(cm & ((1u << lane) - 1u))] = v;
-                dg = (unsigned long long)(__ldg(rowptr + v + 1) - __ldg(rowptr + v));
-            }
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1) dg += __shfl_xor_sync(0xffffffffu, dg, d);
-            if (lane == 0 && dg) atomicAdd(count + 1, dg);
+        int32_t dg = 0;
+        if (claimed) {
+            level[v] = new_level;
+            atomicOr(next + (v >> 5), 1u << (v & 31));
+            dg = __ldg(rowptr + v + 1) - __ldg(rowptr + v);
         }
+        wq.push(claimed, v, dg, next_queue, count);
     }
+    wq.finish(next_queue, count, count + 1);
 }
 
 // ---- cluster-resident push levels ------------------------------------------------------------
