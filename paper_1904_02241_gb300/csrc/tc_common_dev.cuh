@@ -95,10 +95,21 @@ __device__ __forceinline__ T block_sum(T x, T *smem /* >= 32 entries */) {
     return t;
 }
 
+// D / V as the next kernel's threads use it, written beside D by the thread that writes D: this GPU has
+// so little FP64 throughput that a division in every thread showed (20 pull iterations on R-MAT 16: 528
+// to 501 us without it and without the FP64 steps that scaled the sums).
+struct SpreadOut {
+    float *out = nullptr;  // null: not wanted
+    int32_t V = 1;
+    __device__ __forceinline__ void write(double D) const {
+        if (out) *out = (float)(D / (double)V);
+    }
+};
+
 // Every CTA contributes `mine` (valid in thread 0); the last CTA to arrive sums all the
 // contributions in CTA order and stores the total plus `extra` to *out, then re-arms the counter.
 __device__ __forceinline__ void grid_sum_last_cta(double mine, double *part, unsigned *counter, double *out,
-                                                  double extra = 0.0) {
+                                                  double extra = 0.0, SpreadOut spread = SpreadOut()) {
     __shared__ bool am_last;
     __shared__ double red[32];
     if (threadIdx.x == 0) {
@@ -115,6 +126,7 @@ __device__ __forceinline__ void grid_sum_last_cta(double mine, double *part, uns
     t = block_sum<double>(t, red);
     if (threadIdx.x == 0) {
         *out = t + extra;
+        spread.write(t + extra);
         *counter = 0u;
     }
 }
@@ -124,7 +136,8 @@ __device__ __forceinline__ void grid_sum_last_cta(double mine, double *part, uns
 // stores the total to *out and re-arms the counter and *queue (a work queue the CTAs drew from,
 // idle by now: every CTA drew its last item before arriving).  All threads must call it.
 __device__ __forceinline__ void grid_sum_slots_last_cta(const double *part, int32_t nslots, unsigned *counter,
-                                                        unsigned *queue, double *out, double extra = 0.0) {
+                                                        unsigned *queue, double *out, double extra,
+                                                        SpreadOut spread) {
     __shared__ bool am_last3;
     __shared__ double red3[32];
     __syncthreads();
@@ -141,6 +154,7 @@ __device__ __forceinline__ void grid_sum_slots_last_cta(const double *part, int3
     t = block_sum<double>(t, red3);
     if (threadIdx.x == 0) {
         *out = t + extra;
+        spread.write(t + extra);
         *counter = 0u;
         *queue = 0u;
     }

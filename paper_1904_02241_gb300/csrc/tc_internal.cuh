@@ -270,7 +270,7 @@ int32_t tile_max_width(int max_smem_optin);
 // Staged push (tc_push.cu): widest destination range in shared memory, its tiles, the scatter.
 int32_t push_smem_width(int max_smem_optin);
 int build_push_tiles(tc_part *p, int sms, cudaStream_t s);
-int launch_push_smem(const tc_part *p, const float *contrib, void *sums, const double *fx_scale, bool fixed,
+int launch_push_smem(const tc_part *p, const float *contrib, void *sums, const float *fx_scale, bool fixed,
                      cudaStream_t s);
 int build_tiles(tc_part *p, int sms, cudaStream_t s);
 size_t merge_smem_bytes(int32_t k, int32_t B);   // dynamic shared memory of the ordered pull merge

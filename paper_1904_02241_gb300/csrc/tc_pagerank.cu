@@ -20,12 +20,14 @@ struct UpdateArgs {
     int32_t V;
     const double *D_cur;    // dangling mass of the ranks the current contributions came from
     double *D_next;         // dangling mass of the ranks written now
+    const float *S_cur;     // D / V of *D_cur and of *D_next in FP32
+    float *S_next;
     double *dpart;          // per-CTA partial dangling sums
     unsigned *counter;      // arrival counter for the last-CTA reduction
     const float *inv_outdeg;
     float *rank_out;        // may be null (only the last iteration writes ranks)
     float *contrib_next;    // contributions for the next iteration
-    double *fx_scale;       // fixed-point scale of the merge (written by the init kernel)
+    const float *fx_scale;  // fixed-point scale of the sums, a power of two (written by the init kernel)
     const int32_t *perm;    // renumbered partitions: original ID of vertex v (null: identity)
     int32_t nz;             // renumbered: vertices [nz, V) have no out-edges (else nz = V)
     int32_t ni;             // renumbered: vertices [ni, V) have no edge at all (else ni = V)
@@ -40,7 +42,13 @@ struct UpdateArgs {
 };
 
 __device__ __forceinline__ float spread_of(const UpdateArgs &u) {
-    return u.drop ? 0.0f : (float)(*u.D_cur / (double)u.V);
+    return u.drop ? 0.0f : *u.S_cur;
+}
+__device__ __forceinline__ SpreadOut spread_out(const UpdateArgs &u) {
+    SpreadOut o;
+    o.out = u.S_next;
+    o.V = u.V;
+    return o;
 }
 
 // rank[v] = (1-d)/V + d (sum + D/V); contribution = rank / out_degree; returns the dangling share.
@@ -148,7 +156,7 @@ __global__ void __launch_bounds__(PR_THREADS) k_pull_gather(const int32_t *__res
     }
     if (FUSED) {
         const float bs = block_sum<float>(dsum, fred);
-        grid_sum_last_cta((double)bs, u.dpart, u.counter, u.D_next);
+        grid_sum_last_cta((double)bs, u.dpart, u.counter, u.D_next, 0.0, spread_out(u));
     }
 }
 
@@ -314,7 +322,7 @@ __global__ void __launch_bounds__(MG_THREADS) k_pull_merge_ordered(const float *
              v += (int64_t)gridDim.x * MG_THREADS)
             u.rank_out[u.perm ? __ldg(u.perm + v) : v] = r_iso;
     const float bs = block_sum<float>(dsum, fred);
-    grid_sum_last_cta((double)bs, u.dpart, u.counter, u.D_next, (double)(u.V - u.ni) * (double)r_iso);
+    grid_sum_last_cta((double)bs, u.dpart, u.counter, u.D_next, (double)(u.V - u.ni) * (double)r_iso, spread_out(u));
 }
 
 // Rounding to an integer by adding 1.5 * 2^23: for |y| <= 2^22 the sum's low significand
@@ -407,7 +415,7 @@ __global__ void __launch_bounds__(MG_THREADS, 2) k_pull_merge_atomic(const float
     __shared__ int32_t s_next;         // the CTA's next range, drawn from the queue
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // u.fx_scale = 2^61 / mass (a power of two); the parts want 2^44 or 2^48 per unit of mass
-    const float scalef = MODE == 2 ? (float)(*u.fx_scale * 0x1p-17) : (float)(*u.fx_scale * 0x1p-13);
+    const float scalef = *u.fx_scale * (MODE == 2 ? 0x1p-17f : 0x1p-13f);
     const float inv_scalef = 1.0f / scalef;  // a power of two
     const float spread = spread_of(u);
     const bool one = B < MG_THREADS;  // a thread per block (and one for the total): bounds kept in registers
@@ -650,7 +658,8 @@ __global__ void __launch_bounds__(MG_THREADS, 2) k_pull_merge_atomic(const float
         for (int64_t v = (int64_t)u.ni + (int64_t)blockIdx.x * MG_THREADS + tid; v < u.V;
              v += (int64_t)gridDim.x * MG_THREADS)
             u.rank_out[u.perm ? __ldg(u.perm + v) : v] = r_iso;
-    grid_sum_slots_last_cta(u.dpart, nranges, u.counter, u.queue, u.D_next, (double)(u.V - u.ni) * (double)r_iso);
+    grid_sum_slots_last_cta(u.dpart, nranges, u.counter, u.queue, u.D_next,
+                            threadIdx.x == 0 ? (double)(u.V - u.ni) * (double)r_iso : 0.0, spread_out(u));
 }
 
 // Entries per vertex are at most B (one per block): two-part fixed point below 1024 blocks.
@@ -664,7 +673,7 @@ size_t merge_atomic_smem_bytes(int32_t k, int32_t B, bool fixed) {
 // fixed-point scale of the merge: 2^61 / max(1, sum |r|).  No later iteration has a larger
 // L1 mass (each is (1-d) + d * previous at most), so no vertex sum can overflow 2^63.
 __global__ void __launch_bounds__(PR_THREADS) k_pr_init(const float *__restrict__ init, UpdateArgs u, double *mass,
-                                                         double *scale) {
+                                                         float *scale) {
     pdl_wait();  // launched programmatically after the previous call's last kernel
     __shared__ float fred[32];
     float dsum = 0.0f, msum = 0.0f;
@@ -686,7 +695,8 @@ __global__ void __launch_bounds__(PR_THREADS) k_pr_init(const float *__restrict_
         const double m = *mass;
         int e = 0;
         if (m > 1.0) e = (int)ceil(log2(m));
-        *scale = ldexp(1.0, 61 - e);
+        *scale = (float)ldexp(1.0, 61 - e);  // exact: the mass of V finite FP32 values keeps 61 - e above -100
+        spread_out(u).write(*u.D_next);
     }
 }
 
@@ -721,7 +731,7 @@ __device__ __forceinline__ void push_add(void *sums, int32_t d, float c, float s
 
 // The push sums' fixed-point scale: 2^55 per unit of the largest L1 mass, so that |sum| < 2^55
 // (the update converts it with 32-bit steps).
-__device__ __forceinline__ float push_scale(const double *fx_scale) { return (float)(*fx_scale * 0x1p-6); }
+__device__ __forceinline__ float push_scale(const float *fx_scale) { return *fx_scale * 0x1p-6f; }
 
 // Thread/warp/CTA mapping of the rows (Sec. 3.2's TWC): short rows a lane each, rows of at least
 // warp_min edges a warp each, hubs a CTA each.
@@ -732,7 +742,7 @@ __global__ void __launch_bounds__(PR_THREADS) k_push_scatter(const int32_t *__re
                                                              const int32_t *__restrict__ hubs, int32_t num_hubs,
                                                              int32_t hub_degree, int hub_ctas,
                                                              const float *__restrict__ contrib, void *sums,
-                                                             const double *fx_scale, LbArgs lb) {
+                                                             const float *fx_scale, LbArgs lb) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const float scalef = FIXED ? push_scale(fx_scale) : 1.0f;
     if ((int)blockIdx.x < hub_ctas) {
@@ -781,7 +791,7 @@ template <bool FIXED>
 __global__ void __launch_bounds__(PR_THREADS) k_push_edges(const int32_t *__restrict__ esrc,
                                                            const int32_t *__restrict__ dst, int64_t E,
                                                            const float *__restrict__ contrib, void *sums,
-                                                           const double *fx_scale) {
+                                                           const float *fx_scale) {
     const float scalef = FIXED ? push_scale(fx_scale) : 1.0f;
     const int64_t T = (int64_t)gridDim.x * PR_THREADS;
     int64_t i = blockIdx.x * (int64_t)PR_THREADS + threadIdx.x;
@@ -828,7 +838,7 @@ __global__ void __launch_bounds__(PR_THREADS) k_push_update(void *sums, UpdateAr
         dsum += apply_update(u, (int32_t)v, s, spread);
     }
     const float bs = block_sum<float>(dsum, fred);
-    grid_sum_last_cta((double)bs, u.dpart, u.counter, u.D_next);
+    grid_sum_last_cta((double)bs, u.dpart, u.counter, u.D_next, 0.0, spread_out(u));
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -878,10 +888,11 @@ static int occupancy_grid(const void *kernel, int threads, size_t smem, int64_t 
 struct PrState {
     float *contrib[2];
     double *D;          // D[0], D[1]
+    float *S;           // S[0], S[1]: D / V in FP32
     unsigned *counter;
     unsigned *queue;    // work queue of the persistent merge
     double *mass;       // L1 mass of the initial ranks
-    double *scale;      // fixed-point scale of the merge
+    float *scale;       // fixed-point scale of the sums
     int *err;           // sticky error flag of bounded device waits
     double *dpart;      // per-CTA partials (capacity 2 * dpart_cap doubles)
     int64_t dpart_cap;
@@ -906,7 +917,8 @@ static int prepare_state(tc_graph *g, const tc_pr_params *pp, float *ranks_out, 
     st->queue = reinterpret_cast<unsigned *>(sc + 36);
     st->err = reinterpret_cast<int *>(sc + 40);
     st->mass = reinterpret_cast<double *>(sc + 48);
-    st->scale = reinterpret_cast<double *>(sc + 56);
+    st->scale = reinterpret_cast<float *>(sc + 56);
+    st->S = reinterpret_cast<float *>(sc + 16);
     st->dpart = reinterpret_cast<double *>(sc + 128);
     (void)fresh;
     if (pp->out_mem == TC_MEM_DEVICE) {
@@ -1077,6 +1089,8 @@ static int pagerank_impl(const tc_graph *cg, const tc_part *part, const tc_pr_pa
     // init: contributions[0], D[0]
     u.D_cur = st.D + 1;
     u.D_next = st.D + 0;
+    u.S_cur = st.S + 1;
+    u.S_next = st.S + 0;
     u.rank_out = pp->iters == 0 ? st.rank_dev : nullptr;
     u.contrib_next = st.contrib[0];
     {
@@ -1102,6 +1116,8 @@ static int pagerank_impl(const tc_graph *cg, const tc_part *part, const tc_pr_pa
         const float *cur = push ? st.contrib[0] : st.contrib[it & 1];
         u.D_cur = st.D + (it & 1);
         u.D_next = st.D + ((it + 1) & 1);
+        u.S_cur = st.S + (it & 1);
+        u.S_next = st.S + ((it + 1) & 1);
         u.rank_out = last ? st.rank_dev : nullptr;
         u.contrib_next = push ? st.contrib[0] : st.contrib[(it + 1) & 1];
         u.cur = cur;

@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(PS_THREADS, 1) k_push_smem(const int4 *__restr
                                                              const int32_t *__restrict__ esrc,
                                                              const int32_t *__restrict__ dst, int32_t W, int32_t V,
                                                              const float *__restrict__ contrib, void *sums,
-                                                             const double *fx_scale) {
+                                                             const float *fx_scale) {
     extern __shared__ __align__(16) unsigned char psm[];
     unsigned long long *acc64 = reinterpret_cast<unsigned long long *>(psm);
     float *acc32 = reinterpret_cast<float *>(psm);
@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(PS_THREADS, 1) k_push_smem(const int4 *__restr
     const int32_t w = (int32_t)(((int64_t)V - lo) < W ? ((int64_t)V - lo) : W);
     const int64_t e0 = ((int64_t)t.z << 31) | (uint32_t)t.y;  // 62-bit edge bounds split in two ints
     const int64_t e1 = e0 + (uint32_t)t.w;
-    const float scalef = FIXED ? (float)(*fx_scale * 0x1p-6) : 1.0f;  // |sum| < 2^55
+    const float scalef = FIXED ? *fx_scale * 0x1p-6f : 1.0f;  // |sum| < 2^55
     for (int32_t v = threadIdx.x; v < w; v += PS_THREADS) {
         if (FIXED) acc64[v] = 0ull;
         else acc32[v] = 0.0f;
@@ -132,7 +132,7 @@ int build_push_tiles(tc_part *p, int sms, cudaStream_t s) {
     return TC_OK;
 }
 
-int launch_push_smem(const tc_part *p, const float *contrib, void *sums, const double *fx_scale, bool fixed,
+int launch_push_smem(const tc_part *p, const float *contrib, void *sums, const float *fx_scale, bool fixed,
                      cudaStream_t s) {
     if (p->nptiles == 0) return TC_OK;
     const size_t smem = (size_t)p->W * (fixed ? 8 : 4);
