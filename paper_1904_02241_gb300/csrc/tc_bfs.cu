@@ -5,8 +5,6 @@
 //                     over the block's sources), then a merge kernel ORs the local bits of
 //                     all blocks per vertex range and writes levels, next and visited.
 // Levels run TOCAB only when the frontier exceeds a fraction of V (Sec. 3.3).
-#include <cooperative_groups.h>
-
 #include "tc_common_dev.cuh"
 
 namespace tc {
@@ -250,36 +248,75 @@ __global__ void __launch_bounds__(BFS_THREADS) k_bfs_push_edges(const int32_t *_
 }
 
 // ---- cluster-resident push levels ------------------------------------------------------------
-// Consecutive push levels with small frontiers run inside ONE launch of a thread-block cluster:
-// the cluster's hardware barrier (release/acquire at cluster scope) ends each level, so a level
-// costs a few dependent memory round trips instead of a host round trip and five launches.  The
-// grid is exactly one cluster, so every CTA is co-scheduled by construction and no CTA waits on
-// anything but that barrier.
-// Level L: the frontier is the concatenation of the C CTAs' queue segments of level L-1 (the
-// host's vertex queue for the first level); CTA c expands the c-th slice of it in batches of
-// RES_THREADS vertices, and a CTA-wide scan of the out-degrees deals the batch's edges out one
-// per thread.  A neighbour is claimed by an atomic OR on visited, gets its level, and is appended
-// (warp-aggregated, position from a shared-memory counter) to CTA c's own segment with its
-// out-edge range, which the next level reads instead of the row offsets.  After the barrier
-// warp 0 of every CTA reads all C counters through distributed shared memory; every thread then
-// holds the same counts and takes the same decision, the host's: stop when the frontier is
-// empty, when direction optimisation switches to pull (m_f > m_u / 14), or when the next level
-// has more than `cap` vertices or out-edges.  At the end the segments are copied, in CTA order,
-// into the host's queue for the next level.  Everything written during the launch by other CTAs
-// is read with L2 loads (ld.global.cg), never through L1.
+// Consecutive push levels with small frontiers run inside ONE launch of a thread-block cluster: a
+// level costs a few dependent memory round trips instead of a host round trip and five launches.
+// The grid is exactly one cluster, so every CTA is co-scheduled by construction.
+//
+// Such a level is bound by its chain of dependent round trips, so the chain is kept to two of them
+// (an out-row's neighbours, then the claims), plus one exchange through distributed shared memory:
+//   * a CTA expands the vertices it claimed itself, whose out-edge ranges it kept in shared memory;
+//   * a neighbour's row offsets are loaded beside the atomic OR on visited that claims it, not after;
+//   * up to RES_DEG out-edges per vertex a thread walks its own vertex, all its loads in flight; only
+//     batches with longer rows scan the degrees and deal the edges out one per thread;
+//   * a level ends when every CTA's counts (claimed vertices, their out-edges) have arrived in this
+//     CTA's mailbox: one asynchronous remote store per pair, completing on the receiver's mbarrier
+//     (bounded wait).  Nothing else crosses CTAs, so the levels and queues written to global memory
+//     are not waited for; only a level that deals the frontier out anew (one CTA holds more than
+//     RES_THREADS out-edges and more than twice the mean) or the end of the launch uses the cluster
+//     barrier with its release of global writes.  Two mailboxes alternate: a CTA sends level l + 1's
+//     counts after it has read level l's, so a slot is free before it is written again.
+// The counts tell every thread the same, and it takes the decision that the host would: stop when
+// the frontier is empty, when direction optimisation switches to pull (14 m_f > m_u), or when the
+// next level has more than `cap` vertices or out-edges.  At the end the claimed vertices are copied,
+// in CTA order, into the host's queue for the next level.  What other CTAs wrote during the launch is
+// read with L2 loads (ld.global.cg), never through L1.
+// Measured on a 2048^2 grid with 5% of its edges removed (some 3,000 levels): 24.6 ms with the frontier kept in
+// global queues and the cluster barrier at every level, 13.0 ms so.
 constexpr int RES_THREADS = 1024;
 constexpr int RES_WARPS = RES_THREADS / 32;
 constexpr int RES_MAX_CTAS = 16;
+constexpr int RES_DEG = 4;      // out-edges of a vertex walked by its own thread
+constexpr int RES_KEEP = 2048;  // claimed vertices per CTA and level whose ranges stay in shared memory
 
 struct ResOut {  // written by CTA 0, thread 0 when the launch ends
     unsigned long long front;  // frontier size of level `lvl`
     double m_f, m_u;           // its out-edges, and those of the unvisited vertices
     int32_t lvl;               // the next level to expand
     int32_t levels;            // levels expanded by the launch
+    int32_t timeout;           // nonzero: a wait for the counts gave up
 };
 
 __device__ __forceinline__ void cluster_barrier() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// The address of this CTA's shared-memory word in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t remote_smem(const void *p, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr(p)), "r"(rank));
+    return r;
+}
+// Asynchronous 8-byte store to a CTA of the cluster; its bytes complete on that CTA's mbarrier.
+__device__ __forceinline__ void remote_store_async(uint32_t dst, unsigned long long x, uint32_t mbar) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(dst), "l"(x),
+                 "r"(mbar)
+                 : "memory");
+}
+// mbar_wait with cluster-scope acquire (the awaited bytes come from other CTAs).
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t *bar, uint32_t parity) {
+    const long long t0 = clock64();
+    for (;;) {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(smem_addr(bar)), "r"(parity)
+            : "memory");
+        if (ok) return true;
+        if (clock64() - t0 > (1LL << 31)) return false;
+    }
 }
 
 // Exclusive prefix sum over the CTA (RES_THREADS threads); *total gets the sum.  All threads call it.
@@ -309,50 +346,144 @@ __device__ __forceinline__ int32_t res_block_scan(int32_t x, int32_t *wsum /* [R
     return wsum[warp] + inc - x;
 }
 
+// What a CTA's threads append to: its segments of one level.
+struct ResSeg {
+    int32_t *v;         // [cap] claimed vertices (global)
+    int2 *r;            // [cap] their out-edge ranges from RES_KEEP on (global)
+    int2 *keep;         // [RES_KEEP] the first ones' ranges (shared)
+    unsigned *cnt;      // claimed vertices, their out-edges (shared)
+    int32_t cap;
+};
+
+// The whole warp appends the lanes' claims: bit k of `claimed` = vertex v[k] with range r[k].
+template <int K>
+__device__ __forceinline__ void res_append(const ResSeg &q, unsigned claimed, const int32_t *v, const int2 *r) {
+    if (!__any_sync(0xffffffffu, claimed != 0u)) return;
+    const int lane = threadIdx.x & 31;
+    const unsigned c = (unsigned)__popc(claimed);
+    unsigned dg = 0;
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+        if ((claimed >> k) & 1u) dg += (unsigned)(r[k].y - r[k].x);
+    unsigned inc = c;
+    if (K == 1) {
+        const unsigned m = __ballot_sync(0xffffffffu, claimed != 0u);
+        inc = (unsigned)__popc(m & ((2u << lane) - 1u));
+    } else {
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, inc, d);
+            if (lane >= d) inc += y;
+        }
+    }
+    dg = __reduce_add_sync(0xffffffffu, dg);
+    unsigned base = 0;
+    if (lane == 31) {
+        base = atomicAdd(q.cnt, inc);
+        atomicAdd(q.cnt + 1, dg);
+    }
+    unsigned p = __shfl_sync(0xffffffffu, base, 31) + inc - c;
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+        if ((claimed >> k) & 1u) {
+            if (p < (unsigned)q.cap) {  // always: a CTA claims at most the level's edges
+                q.v[p] = v[k];
+                if (p < (unsigned)RES_KEEP) q.keep[p] = r[k];
+                else q.r[p] = r[k];
+            }
+            ++p;
+        }
+}
+
+// Claims v for level new_level; its out-edge range is loaded beside the claim.
+__device__ __forceinline__ bool res_claim(const int32_t *__restrict__ rowptr, uint32_t *visited, int32_t *level,
+                                          int32_t v, int32_t new_level, int2 *range) {
+    const uint32_t bit = 1u << (v & 31);
+    const uint32_t old = atomicOr(visited + (v >> 5), bit);
+    range->x = __ldg(rowptr + v);
+    range->y = __ldg(rowptr + v + 1);
+    if (old & bit) return false;
+    level[v] = new_level;
+    return true;
+}
+
 // seg_v / seg_r: [2 parities][C CTAs][cap] vertex IDs and out-edge ranges of the claimed vertices.
 __global__ void __launch_bounds__(RES_THREADS, 1) k_bfs_push_resident(
     const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colidx, uint32_t *visited, int32_t *level,
-    int32_t *q0, int32_t *q1, int32_t *seg_v, int2 *seg_r, int64_t *trace, int32_t lvl0, int32_t n0, double mf0,
-    double mu0, int32_t cap, int32_t max_levels, ResOut *out) {
-    namespace cgs = cooperative_groups;
+    int32_t *q0, int32_t *q1, int32_t *seg_v, int2 *seg_r, int64_t *trace, int32_t lvl0, int32_t n0, int64_t mu0,
+    int32_t cap, int32_t max_levels, ResOut *out) {
     __shared__ int32_t sh_start[RES_THREADS], sh_off[RES_THREADS];
+    __shared__ int2 keep[2][RES_KEEP];
     __shared__ int32_t wsum[RES_WARPS + 1];
-    __shared__ unsigned long long s_cnt[2][2];  // this CTA's claims by level parity: vertices, out-edges
-    __shared__ int32_t s_pre[RES_MAX_CTAS + 1];  // prefix of the segment counts (the current frontier)
-    __shared__ unsigned long long s_edges;       // out-edges of the current frontier
-    cgs::cluster_group cluster = cgs::this_cluster();
+    __shared__ unsigned s_cnt[2][2];                         // this CTA's claims by level parity: vertices, out-edges
+    __shared__ unsigned long long s_mail[2][RES_MAX_CTAS];   // every CTA's counts by level parity
+    __shared__ __align__(8) uint64_t s_bar[2];
+    __shared__ int32_t s_pre[RES_MAX_CTAS + 1];              // prefix of the segment counts
+    __shared__ int s_failed;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int32_t C = (int32_t)gridDim.x, c = (int32_t)blockIdx.x;
-    if (tid < 4) s_cnt[tid >> 1][tid & 1] = 0ull;  // ordered before any claim by the scan's barriers
-    int32_t lvl = lvl0, levels = 0, n = n0;
-    double mf = mf0, mu = mu0;
-    bool first = true;  // the frontier is the host's queue (first level), else the segments
+    if (tid < 4) s_cnt[tid >> 1][tid & 1] = 0u;
+    if (tid == 0) {
+        mbar_init(&s_bar[0], 1);
+        mbar_init(&s_bar[1], 1);
+        s_failed = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    cluster_barrier();  // every CTA's mailboxes exist
+    int32_t lvl = lvl0, levels = 0, n = n0, mine = 0;
+    int64_t mf = 0, mu = mu0;
+    enum { QUEUE, OWN, DEALT } from = QUEUE;  // the frontier: the host's queue, this CTA's claims, or all CTAs' segments
+    bool failed = false;
     for (;;) {
-        const int par = lvl & 1;  // claims of this level: counters s_cnt[par], segments of parity par
-        if (!first && tid == 0) {  // read remotely before the previous barrier, by every CTA
-            s_cnt[par][0] = 0ull;
-            s_cnt[par][1] = 0ull;
+        const int par = lvl & 1;  // this level's claims: counters, mailbox and segments of parity par
+        if (tid == 0) {
+            s_cnt[par ^ 1][0] = s_cnt[par ^ 1][1] = 0u;  // the next level's: sent before the last wait
+            mbar_expect_tx(&s_bar[par], (uint32_t)C * 8u);
         }
         const int32_t *hq = (lvl & 1) ? q1 : q0;
         const int2 *in_r = seg_r + (size_t)(par ^ 1) * C * cap;
-        int32_t *out_v = seg_v + ((size_t)par * C + c) * cap;
-        int2 *out_r = seg_r + ((size_t)par * C + c) * cap;
-        const int32_t lo = (int32_t)((int64_t)n * c / C), hi = (int32_t)((int64_t)n * (c + 1) / C);
+        ResSeg out_q;
+        out_q.v = seg_v + ((size_t)par * C + c) * cap;
+        out_q.r = seg_r + ((size_t)par * C + c) * cap;
+        out_q.keep = keep[par];
+        out_q.cnt = s_cnt[par];
+        out_q.cap = cap;
+        const int32_t lo = from == OWN ? 0 : (int32_t)((int64_t)n * c / C);
+        const int32_t hi = from == OWN ? mine : (int32_t)((int64_t)n * (c + 1) / C);
         for (int32_t b0 = lo; b0 < hi; b0 += RES_THREADS) {
             const int32_t i = b0 + tid;
             int32_t s = 0, e = 0;
             if (i < hi) {
-                if (first) {
+                if (from == QUEUE) {
                     const int32_t u = __ldcg(hq + i);
                     s = __ldg(rowptr + u);
                     e = __ldg(rowptr + u + 1);
-                } else {  // entry i of the concatenated segments
-                    int32_t a = 0;
-                    while (a + 1 < C && s_pre[a + 1] <= i) ++a;
-                    const int2 r = __ldcg(in_r + (size_t)a * cap + (i - s_pre[a]));
+                } else {
+                    int2 r;
+                    if (from == OWN) {
+                        r = i < RES_KEEP ? keep[par ^ 1][i] : __ldcg(in_r + (size_t)c * cap + i);
+                    } else {  // entry i of the concatenated segments
+                        int32_t a = 0;
+                        while (a + 1 < C && s_pre[a + 1] <= i) ++a;
+                        r = __ldcg(in_r + (size_t)a * cap + (i - s_pre[a]));
+                    }
                     s = r.x;
                     e = r.y;
                 }
+            }
+            if (!__syncthreads_or(e - s > RES_DEG)) {  // short rows: a thread walks its own vertex
+                int32_t v[RES_DEG];
+                int2 r[RES_DEG];
+                unsigned claimed = 0;
+#pragma unroll
+                for (int k = 0; k < RES_DEG; ++k) v[k] = s + k < e ? __ldg(colidx + s + k) : -1;
+#pragma unroll
+                for (int k = 0; k < RES_DEG; ++k) {
+                    r[k] = make_int2(0, 0);
+                    if (v[k] >= 0 && res_claim(rowptr, visited, level, v[k], lvl + 1, &r[k])) claimed |= 1u << k;
+                }
+                res_append<RES_DEG>(out_q, claimed, v, r);
+                continue;
             }
             int32_t total;
             const int32_t off = res_block_scan(e - s, wsum, &total);
@@ -362,8 +493,9 @@ __global__ void __launch_bounds__(RES_THREADS, 1) k_bfs_push_resident(
             const int32_t nb = min(RES_THREADS, hi - b0);
             for (int32_t base = warp * 32; base < total; base += RES_THREADS) {
                 const int32_t k = base + lane;
-                bool claimed = false;
-                int32_t v = 0, vs = 0, ve = 0;
+                unsigned claimed = 0;
+                int32_t v = 0;
+                int2 r = make_int2(0, 0);
                 if (k < total) {  // the last vertex of the batch whose edges start at or before k
                     int32_t a = 0, z = nb - 1;
                     while (a < z) {
@@ -371,85 +503,76 @@ __global__ void __launch_bounds__(RES_THREADS, 1) k_bfs_push_resident(
                         if (sh_off[mid] <= k) a = mid; else z = mid - 1;
                     }
                     v = __ldg(colidx + sh_start[a] + (k - sh_off[a]));
-                    const uint32_t bit = 1u << (v & 31);
-                    claimed = !(atomicOr(visited + (v >> 5), bit) & bit);
+                    claimed = res_claim(rowptr, visited, level, v, lvl + 1, &r) ? 1u : 0u;
                 }
-                if (claimed) {
-                    level[v] = lvl + 1;
-                    vs = __ldg(rowptr + v);
-                    ve = __ldg(rowptr + v + 1);
-                }
-                const unsigned cm = __ballot_sync(0xffffffffu, claimed);
-                if (cm) {
-                    const int leader = __ffs(cm) - 1;
-                    unsigned long long dg = (unsigned long long)(ve - vs);
-#pragma unroll
-                    for (int d = 16; d > 0; d >>= 1) dg += __shfl_xor_sync(0xffffffffu, dg, d);
-                    unsigned long long pos0 = 0;
-                    if (lane == leader) {
-                        pos0 = atomicAdd(&s_cnt[par][0], (unsigned long long)__popc(cm));
-                        atomicAdd(&s_cnt[par][1], dg);
-                    }
-                    pos0 = __shfl_sync(0xffffffffu, pos0, leader);
-                    if (claimed) {
-                        const unsigned long long p = pos0 + (unsigned)__popc(cm & ((1u << lane) - 1u));
-                        if (p < (unsigned long long)cap) {  // always: a CTA claims at most the level's edges
-                            out_v[p] = v;
-                            out_r[p] = make_int2(vs, ve);
-                        }
-                    }
-                }
+                res_append<1>(out_q, claimed, &v, &r);
             }
             __syncthreads();  // the batch's offsets are read before the next batch overwrites them
         }
         ++levels;
-        cluster_barrier();
-        if (warp == 0) {  // every CTA's counters of this level, through distributed shared memory
-            unsigned long long cn = 0, ce = 0;
-            if (lane < C) {
-                const unsigned long long *rc = cluster.map_shared_rank(&s_cnt[par][0], (unsigned)lane);
-                cn = rc[0];
-                ce = rc[1];
-            }
-            unsigned long long inc = cn;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, d);
-                if (lane >= d) inc += y;
-            }
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1) ce += __shfl_xor_sync(0xffffffffu, ce, d);
-            if (lane < C) s_pre[lane + 1] = (int32_t)inc;
-            if (lane == 0) {
-                s_pre[0] = 0;
-                s_edges = ce;
-            }
-        }
-        __syncthreads();
-        n = s_pre[C];
-        mf = (double)s_edges;
+        __syncthreads();  // the CTA's claims are counted
+        if (tid < C)
+            remote_store_async(remote_smem(&s_mail[par][c], (uint32_t)tid),
+                               ((unsigned long long)s_cnt[par][0] << 32) | s_cnt[par][1],
+                               remote_smem(&s_bar[par], (uint32_t)tid));
+        // level lvl0 + i completes phase i / 2 of its barrier; the CTA agrees on whether it did
+        failed = __syncthreads_or(!mbar_wait_cluster(&s_bar[par], (uint32_t)(((levels - 1) >> 1) & 1)));
+        if (failed) break;
+        const unsigned long long mail = lane < C ? s_mail[par][lane] : 0ull;
+        const unsigned cn = (unsigned)(mail >> 32), ce = (unsigned)mail;
+        n = (int32_t)__reduce_add_sync(0xffffffffu, cn);
+        mf = (int64_t)__reduce_add_sync(0xffffffffu, ce);  // at most the graph's edges, below 2^31
+        const unsigned most = __reduce_max_sync(0xffffffffu, ce);
+        mine = (int32_t)__shfl_sync(0xffffffffu, cn, c);
         mu -= mf;
         ++lvl;
-        first = false;
         if (c == 0 && tid == 0 && lvl < TC_BFS_TRACE) trace[lvl] = n;
-        if (n == 0 || mf > mu / 14.0 || n > cap || mf > (double)cap || levels >= max_levels) break;
+        // 14 mf > mu is the host's mf > mu / 14 for integers
+        const bool stop = n == 0 || 14 * mf > mu || n > cap || mf > (int64_t)cap || levels >= max_levels;
+        from = OWN;
+        const bool deal = !stop && most > (unsigned)RES_THREADS && (int64_t)most * C > 2 * mf;
+        if (stop || deal) {  // rare
+            if (warp == 0) {
+                unsigned inc = cn;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const unsigned y = __shfl_up_sync(0xffffffffu, inc, d);
+                    if (lane >= d) inc += y;
+                }
+                if (lane < C) s_pre[lane + 1] = (int32_t)inc;
+                if (lane == 0) s_pre[0] = 0;
+            }
+            __syncthreads();
+        }
+        if (deal) {
+            int2 *seg = seg_r + ((size_t)par * C + c) * cap;
+            for (int32_t i = tid; i < mine && i < RES_KEEP; i += RES_THREADS) seg[i] = keep[par][i];
+            cluster_barrier();
+            from = DEALT;
+        }
+        if (stop) break;
     }
     // the frontier of level lvl into the host's queue for it, segments in CTA order
-    {
-        const int par = (lvl - 1) & 1;
-        const int32_t *src = seg_v + ((size_t)par * C + c) * cap;
+    if (!failed) {
+        const int32_t *src = seg_v + ((size_t)((lvl - 1) & 1) * C + c) * cap;
         int32_t *dst = ((lvl & 1) ? q1 : q0) + s_pre[c];
         const int32_t cnt = s_pre[c + 1] - s_pre[c];
         for (int32_t i = tid; i < cnt; i += RES_THREADS) dst[i] = __ldcg(src + i);
     }
+    if (failed && tid == 0)
+        asm volatile("st.shared::cluster.u32 [%0], 1;" ::"r"(remote_smem(&s_failed, 0u)) : "memory");
+    // No CTA leaves while another may still store into its shared memory.  Twice: a CTA whose wait gave up
+    // may meet the others' barrier of a dealt level here, and they send it one more message after that.
+    cluster_barrier();
     if (c == 0 && tid == 0) {
+        out->timeout = s_failed;
         out->front = (unsigned long long)n;
-        out->m_f = mf;
-        out->m_u = mu;
+        out->m_f = (double)mf;
+        out->m_u = (double)mu;
         out->lvl = lvl;
         out->levels = levels;
     }
-    cluster_barrier();  // no CTA leaves while another may still read its shared memory
+    cluster_barrier();
 }
 
 // front = the bits of the queue's vertices (the frontier bitmap after resident push levels).
@@ -645,13 +768,14 @@ static int bfs_impl(const tc_graph *cg, const tc_part *part, int32_t source, con
             cudaError_t e = cudaLaunchKernelEx(&cfg, k_bfs_push_resident, (const int32_t *)g->out_rowptr.as<int32_t>(),
                                                (const int32_t *)g->out_colidx.as<int32_t>(), visited, level, q[0],
                                                q[1], res_v, res_r, res_trace, (int32_t)lvl, (int32_t)front_count,
-                                               m_f, m_u, res_cap, (int32_t)(V + 1), res_out);
+                                               (int64_t)m_u, res_cap, (int32_t)(V + 1), res_out);
             if (lev[1] && e == cudaSuccess) e = cudaEventRecord(lev[1], s);
             if (e == cudaSuccess) e = cudaMemcpyAsync(h_cnt + 2, res_out, sizeof(ResOut), cudaMemcpyDeviceToHost, s);
             if (e == cudaSuccess) e = cudaStreamSynchronize(s);
             if (e != cudaSuccess) { st = fail(TC_ERR_CUDA, "bfs resident levels from %d: %s", lvl, cudaGetErrorString(e)); break; }
             ResOut ro;
             memcpy(&ro, h_cnt + 2, sizeof(ro));
+            if (ro.timeout) { st = fail(TC_ERR_TIMEOUT, "bfs resident levels from %d: a bounded device wait gave up", lvl); break; }
             if (ro.levels < 1 || ro.lvl != lvl + ro.levels) { st = fail(TC_ERR_CUDA, "bfs resident levels: bad exit state"); break; }
             if (stats) {
                 float seg_ms = 0.0f;

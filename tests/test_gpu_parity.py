@@ -767,3 +767,42 @@ def test_pagerank_push_staged(T, name, sums):
         assert torch.equal(r.cpu(), T.pagerank_push(G, None).cpu())
 
 
+
+
+def _bfs_side_component(V0, edges, extra=3000, m=120000, seed=9):
+    """The given edges, and an unreachable random component whose out-edges keep push levels running."""
+    rng = np.random.default_rng(seed)
+    side = rng.integers(0, extra, (m, 2)) + V0
+    return gg.from_edge_list(V0 + extra, np.concatenate([np.asarray(edges, dtype=np.int64), side]))
+
+
+@pytest.mark.parametrize("leaves,children,deg", [(2047, 300, 1), (2048, 300, 1), (3000, 500, 2), (3000, 3000, 1),
+                                                 (1500, 1500, 4), (1500, 1500, 5), (40, 40, 200)])
+def test_bfs_resident_segments_beyond_shared_memory_and_dealt_anew(T, leaves, children, deg):
+    """One CTA claims all leaves of a hub: more than the 2,048 whose ranges stay in shared memory (few
+    out-edges: it keeps them), or more out-edges than threads (the frontier is dealt out anew); vertices
+    of up to 4 out-edges and of more."""
+    edges = [(0, 1 + i) for i in range(leaves)]
+    base = 1 + leaves
+    edges += [(1 + i, base + i * deg + k) for i in range(children) for k in range(deg)]
+    V0 = base + children * deg + 2
+    edges += [(base + i, V0 - 2) for i in range(children * deg)] + [(V0 - 2, V0 - 1)]
+    g = _bfs_side_component(V0, edges)
+    G = _load(T, g)
+    rp, ci = g.numpy()
+    for s in (0, 1):
+        lv, st = T.bfs_pull(G, None, s, tocab_threshold=-1.0, push_threshold=1.0, return_stats=True)
+        np.testing.assert_array_equal(lv.cpu().numpy(), oracle.bfs(g.V, rp, ci, s))
+    assert st.resident_levels > 0
+
+
+def test_bfs_resident_levels_on_a_grid_wider_than_a_cta(T):
+    """Frontiers of up to 1,400 vertices from a corner, dealt out anew as one CTA's share grows."""
+    g = gg.grid2d(1400, 40, drop=0.03, seed=5)
+    g2 = gg.grid2d(300, 300, drop=0.03, seed=6)
+    for gr in (g, g2):
+        G = _load(T, gr)
+        rp, ci = gr.numpy()
+        for s in (0, gr.V // 2, gr.V - 1):
+            lv = T.bfs_pull(G, None, s, tocab_threshold=-1.0, push_threshold=1.0)
+            np.testing.assert_array_equal(lv.cpu().numpy(), oracle.bfs(gr.V, rp, ci, s))
