@@ -806,3 +806,24 @@ def test_bfs_resident_levels_on_a_grid_wider_than_a_cta(T):
         for s in (0, gr.V // 2, gr.V - 1):
             lv = T.bfs_pull(G, None, s, tocab_threshold=-1.0, push_threshold=1.0)
             np.testing.assert_array_equal(lv.cpu().numpy(), oracle.bfs(gr.V, rp, ci, s))
+
+
+@pytest.mark.parametrize("name,B", [("rmat15", 1), ("rmat15", 3), ("rmat15", 8), ("rmat15", 100), ("er", 2), ("er", 7),
+                                    ("islands", 5)])
+def test_bfs_blocked_levels_from_shared_memory(T, name, B):
+    """Blocked levels over several 8,192-row chunks: chunks inside one block (its bitmap slice in shared
+    memory, with and without frontier vertices) and across block ends, streamed and early-exit levels."""
+    if name == "islands":  # half of the blocks never hold a frontier vertex
+        a = gg.symmetrize(gg.rmat(13)).numpy()
+        e = np.stack([np.repeat(np.arange(1 << 13), np.diff(a[0])), a[1]], 1)
+        g = gg.from_edge_list(3 << 13, np.concatenate([e, e + (2 << 13)]))
+    else:
+        g = {"rmat15": lambda: gg.symmetrize(gg.rmat(15)),
+             "er": lambda: gg.symmetrize(gg.erdos_renyi(50001, 200000, seed=8))}[name]()
+    G = _load(T, g)
+    P = T.tocab_partition(G, T.TC_PULL, B, smem_stage=-1)
+    rp, ci = g.numpy()
+    for s in gg.sources(g, 2, seed=41):
+        lv, st = T.bfs_pull(G, P, s, tocab_threshold=0.0, return_stats=True)
+        np.testing.assert_array_equal(lv.cpu().numpy(), oracle.bfs(g.V, rp, ci, s))
+        assert st.tocab_levels == st.levels
