@@ -25,7 +25,11 @@
 // vertex's dependency reads only final values of the next level, so the order of a level's list
 // (which the forward sweep fills as vertices are reached) does not change any result.
 //
-// sigma, the coefficients and the scores are FP64.
+// sigma, the coefficients and the scores are FP64.  The coefficients are kept in two arrays by the parity
+// of the vertex's depth, zero in the other one, so that an edge of the backward sweep reads one value
+// and no depth: a vertex of depth L that reads the array of parity L+1 meets nonzero values at depth
+// L+1 only (no out-edge spans two levels, and shallower levels have no coefficients yet), and adding
+// the zeros of the others changes no sum.
 #include <vector>
 
 #include "tc_common_dev.cuh"
@@ -36,11 +40,69 @@ constexpr int BC_THREADS = 256;
 constexpr int BC_WARPS = BC_THREADS / 32;
 constexpr int BC_LONG = 32;  // rows with at least this many edges get a warp in pull levels
 
-__global__ void k_bc_init(int32_t V, int32_t source, int32_t *depth, double *sigma, double *coef, int32_t *order) {
+struct BcPair {  // one array per parity of the depth
+    double *even, *odd;
+    __host__ __device__ __forceinline__ double *at(int32_t L) const { return (L & 1) ? odd : even; }
+};
+
+// This lane's share of a row: x of the columns first, first + step, ... below e, added in order; with
+// `depth`, of those of depth L only.  The whole warp calls it (a lane without a row passes an empty one).
+// Two things bound a row.  One load at a time, it is a chain of dependent round trips, and a level waits
+// for its longest one (a hub's share of its CTA), so up to U loads of each kind are in flight.  And an
+// FP64 addition takes its SM some 16 cycles per warp however few lanes need it, so a lane skips to its
+// next nonzero value and the warp adds as often as its fullest lane needs (tested on the bits: comparing
+// doubles is FP64 work too).
+constexpr unsigned FULL_WARP = 0xffffffffu;
+__device__ __forceinline__ bool bc_any(double x) { return __any_sync(FULL_WARP, __double_as_longlong(x) != 0ll); }
+
+template <int U>
+__device__ __forceinline__ double bc_row_sum(const int32_t *__restrict__ colidx, int32_t first, int32_t e, int32_t step,
+                                             const double *x, const int32_t *depth = nullptr, int32_t L = 0) {
+    double t = 0.0;
+    for (int64_t i = first; __any_sync(FULL_WARP, i < e); i += (int64_t)U * step) {
+        int32_t c[U];
+        double y[U];
+#pragma unroll
+        for (int k = 0; k < U; ++k) c[k] = i + (int64_t)k * step < e ? __ldg(colidx + i + (int64_t)k * step) : -1;
+        if (depth) {
+            int32_t d[U];
+#pragma unroll
+            for (int k = 0; k < U; ++k) d[k] = c[k] >= 0 ? depth[c[k]] : -1;
+#pragma unroll
+            for (int k = 0; k < U; ++k)
+                if (d[k] != L) c[k] = -1;
+        }
+#pragma unroll
+        for (int k = 0; k < U; ++k) y[k] = c[k] >= 0 ? x[c[k]] : 0.0;
+        unsigned m = 0;  // this lane's nonzero values, added lowest first
+#pragma unroll
+        for (int k = 0; k < U; ++k) m |= __double_as_longlong(y[k]) != 0ll ? 1u << k : 0u;
+        while (__any_sync(FULL_WARP, m != 0u)) {
+            double z = 0.0;
+#pragma unroll
+            for (int k = U - 1; k >= 0; --k)
+                if ((m >> k) & 1u) z = y[k];
+            m &= m - 1u;
+            t = __dadd_rn(t, z);
+        }
+    }
+    return t;
+}
+
+// The lanes' shares in a fixed tree over groups of G lanes; every lane of the group gets the sum.
+template <int G>
+__device__ __forceinline__ double bc_group_sum(double t) {
+    if (bc_any(t)) {
+#pragma unroll
+        for (int q = G / 2; q > 0; q >>= 1) t = __dadd_rn(t, __shfl_xor_sync(FULL_WARP, t, q));
+    }
+    return t;
+}
+
+__global__ void k_bc_init(int32_t V, int32_t source, int32_t *depth, double *sigma, int32_t *order) {
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < V; v += (int64_t)gridDim.x * blockDim.x) {
         depth[v] = v == source ? 0 : -1;
         sigma[v] = v == source ? 1.0 : 0.0;
-        coef[v] = 0.0;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) order[0] = source;  // level 0
 }
@@ -122,11 +184,7 @@ __global__ void __launch_bounds__(BC_THREADS) k_bc_pull(const int32_t *__restric
         const int32_t v = hubs[blockIdx.x];
         const bool open = depth[v] == -1;  // the same for the whole CTA: only this CTA sets it
         double acc = 0.0;
-        if (open)
-            for (int32_t i = in_rowptr[v] + threadIdx.x; i < in_rowptr[v + 1]; i += BC_THREADS) {
-                const int32_t u = in_colidx[i];
-                if (depth[u] == L) acc = __dadd_rn(acc, sigma[u]);
-            }
+        if (open) acc = bc_row_sum<8>(in_colidx, in_rowptr[v] + threadIdx.x, in_rowptr[v + 1], BC_THREADS, sigma, depth, L);
         acc = block_sum<double>(acc, red);  // every thread has read depth[v] by now
         const bool hit = open && acc != 0.0 && threadIdx.x == 0;  // sigma of a reached vertex is at least 1
         if (hit) {
@@ -144,27 +202,16 @@ __global__ void __launch_bounds__(BC_THREADS) k_bc_pull(const int32_t *__restric
                 e = in_rowptr[v + 1];
                 if (e - s > hub_degree) e = s;  // its own CTA
             }
-            double acc = 0.0;
-            if (e - s < BC_LONG)
-                for (int32_t i = s; i < e; ++i) {
-                    const int32_t u = in_colidx[i];
-                    if (depth[u] == L) acc = __dadd_rn(acc, sigma[u]);
-                }
+            double acc = bc_row_sum<4>(in_colidx, s, e - s < BC_LONG ? e : s, 1, sigma, depth, L);
             unsigned long_rows = __ballot_sync(0xffffffffu, e - s >= BC_LONG);
             while (long_rows) {
                 const int l = __ffs(long_rows) - 1;
                 long_rows &= long_rows - 1;
                 const int32_t ls = __shfl_sync(0xffffffffu, s, l), le = __shfl_sync(0xffffffffu, e, l);
-                double w = 0.0;
-                for (int32_t i = ls + lane; i < le; i += 32) {
-                    const int32_t u = in_colidx[i];
-                    if (depth[u] == L) w = __dadd_rn(w, sigma[u]);
-                }
-#pragma unroll
-                for (int d = 16; d > 0; d >>= 1) w = __dadd_rn(w, __shfl_xor_sync(0xffffffffu, w, d));
+                const double w = bc_group_sum<32>(bc_row_sum<8>(in_colidx, ls + lane, le, 32, sigma, depth, L));
                 if (lane == l) acc = w;
             }
-            const bool hit = acc != 0.0;
+            const bool hit = __double_as_longlong(acc) != 0ll;
             if (hit) {
                 depth[v] = L + 1;
                 sigma[v] = acc;
@@ -194,24 +241,13 @@ __global__ void __launch_bounds__(BC_THREADS) k_bc_block_level(const int32_t *__
             s = __ldg(rowptr + r);
             e = __ldg(rowptr + r + 1);
         }
-        double acc = 0.0;
-        if (e - s < BC_LONG)
-            for (int32_t i = s; i < e; ++i) {
-                const int32_t u = __ldg(colidx + i);
-                if (depth[u] == L) acc = __dadd_rn(acc, sigma[u]);
-            }
+        double acc = bc_row_sum<4>(colidx, s, e - s < BC_LONG ? e : s, 1, sigma, depth, L);
         unsigned long_rows = __ballot_sync(0xffffffffu, e - s >= BC_LONG);
         while (long_rows) {
             const int l = __ffs(long_rows) - 1;
             long_rows &= long_rows - 1;
             const int32_t ls = __shfl_sync(0xffffffffu, s, l), le = __shfl_sync(0xffffffffu, e, l);
-            double w = 0.0;
-            for (int32_t i = ls + lane; i < le; i += 32) {
-                const int32_t u = __ldg(colidx + i);
-                if (depth[u] == L) w = __dadd_rn(w, sigma[u]);
-            }
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1) w = __dadd_rn(w, __shfl_xor_sync(0xffffffffu, w, d));
+            const double w = bc_group_sum<32>(bc_row_sum<8>(colidx, ls + lane, le, 32, sigma, depth, L));
             if (lane == l) acc = w;
         }
         if (r < R) partial[r] = acc;
@@ -277,66 +313,74 @@ __device__ __forceinline__ void bc_dep_update(int32_t v, double t, int32_t sourc
 // them the warp that met the vertex.  Each class adds in a fixed order, so scores repeat bit for bit.
 // One launch per level instead of one per class, which read the level's list twice and cost three
 // launches on the small levels (4 sources on a symmetrised R-MAT 18: 1,077 us of 2,096 in 75 launches).
+// Bound by FP64 instructions where rows have many children, else by the longest row a warp meets.  With
+// batched loads, skipped zeros, 32 divisions at a time and one vertex per warp step on all but the largest
+// levels: 4 sources on a symmetrised R-MAT 18 1,702 to 1,422 us (the sweep's largest level 103 to 53 us).
 constexpr int32_t BC_SMALL = 64;
 
 __global__ void __launch_bounds__(BC_THREADS) k_bc_backward(const int32_t *__restrict__ rowptr,
                                                             const int32_t *__restrict__ colidx,
                                                             const int32_t *__restrict__ level_list, int64_t n,
                                                             const int32_t *__restrict__ hubs, int32_t nhubs, int32_t L,
-                                                            int32_t source, int32_t small_max, int32_t hub_degree,
+                                                            int32_t source, int32_t small_max, int32_t hub_degree, int32_t per,
                                                             const int32_t *__restrict__ depth,
-                                                            const double *__restrict__ sigma, double *coef,
+                                                            const double *__restrict__ sigma,
+                                                            const double *coef_next, double *coef,
                                                             double *score) {
     __shared__ double red[32];
     if ((int32_t)blockIdx.x < nhubs) {
         const int32_t v = hubs[blockIdx.x];
         if (depth[v] != L) return;  // the same for the whole CTA
-        double t = 0.0;
-        for (int32_t e = rowptr[v] + threadIdx.x; e < rowptr[v + 1]; e += BC_THREADS) {
-            const int32_t w = colidx[e];
-            if (depth[w] == L + 1) t = __dadd_rn(t, coef[w]);
-        }
+        double t = bc_row_sum<8>(colidx, rowptr[v] + threadIdx.x, rowptr[v + 1], BC_THREADS, coef_next);
         t = block_sum<double>(t, red);
         if (threadIdx.x == 0) bc_dep_update(v, t, source, sigma, coef, score);
         return;
     }
-    const int lane = threadIdx.x & 31, sub = lane & 7;
-    const int64_t step = (int64_t)(gridDim.x - nhubs) * BC_WARPS * 4;
-    // warp-uniform loop: the shuffles below see the whole warp
-    for (int64_t base = (((int64_t)(blockIdx.x - nhubs) * BC_THREADS + threadIdx.x) >> 5) * 4; base < n; base += step) {
+    // the vertices' sums wait here until 32 of them take their divisions together: one update per four
+    // vertices kept the FP64 unit busy with four lanes of a warp
+    __shared__ double wait_t[BC_WARPS][32];
+    __shared__ int32_t wait_v[BC_WARPS][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane & 7;
+    int nwait = 0;  // warp-uniform, at most 28 before a step
+    // `per` vertices at a time (4 or 1), neighbours in the list to different CTAs: a level's long rows
+    // stand close together in it, and are walked one after the other by the warp that meets them
+    const int64_t ctas = gridDim.x - nhubs, step = ctas * BC_WARPS * per;
+    // warp-uniform loop: the votes and shuffles below see the whole warp
+    for (int64_t base = ((int64_t)warp * ctas + (blockIdx.x - nhubs)) * per; base < n; base += step) {
         const int64_t k = base + (lane >> 3);
         int32_t v = -1, s = 0, e = 0;
-        if (k < n) {
+        if ((lane >> 3) < per && k < n) {
             v = level_list[k];
             s = rowptr[v];
             e = rowptr[v + 1];
         }
         const bool small = e - s <= small_max;
-        double t = 0.0;
-        if (small)
-            for (int32_t i = s + sub; i < e; i += 8) {
-                const int32_t w = colidx[i];
-                if (depth[w] == L + 1) t = __dadd_rn(t, coef[w]);
-            }
-#pragma unroll
-        for (int q = 4; q > 0; q >>= 1) t = __dadd_rn(t, __shfl_xor_sync(0xffffffffu, t, q));
-        if (sub == 0 && v >= 0 && small) bc_dep_update(v, t, source, sigma, coef, score);
-        unsigned wm = __ballot_sync(0xffffffffu, sub == 0 && !small && e - s <= hub_degree);
+        double t = bc_group_sum<8>(bc_row_sum<4>(colidx, s + sub, small ? e : s, 8, coef_next));
+        unsigned wm = __ballot_sync(FULL_WARP, sub == 0 && !small && e - s <= hub_degree);
         while (wm) {
             const int l = __ffs(wm) - 1;
             wm &= wm - 1;
-            const int32_t lv = __shfl_sync(0xffffffffu, v, l);
-            const int32_t ls = __shfl_sync(0xffffffffu, s, l), le = __shfl_sync(0xffffffffu, e, l);
-            double x = 0.0;
-            for (int32_t i = ls + lane; i < le; i += 32) {
-                const int32_t w = colidx[i];
-                if (depth[w] == L + 1) x = __dadd_rn(x, coef[w]);
-            }
-#pragma unroll
-            for (int q = 16; q > 0; q >>= 1) x = __dadd_rn(x, __shfl_xor_sync(0xffffffffu, x, q));
-            if (lane == 0) bc_dep_update(lv, x, source, sigma, coef, score);
+            const int32_t ls = __shfl_sync(FULL_WARP, s, l), le = __shfl_sync(FULL_WARP, e, l);
+            const double x = bc_group_sum<32>(bc_row_sum<8>(colidx, ls + lane, le, 32, coef_next));
+            if (lane == l) t = x;
+        }
+        const bool done = sub == 0 && v >= 0 && e - s <= hub_degree;
+        const unsigned m = __ballot_sync(FULL_WARP, done);
+        if (done) {
+            const int at = nwait + __popc(m & ((1u << lane) - 1u));
+            wait_t[warp][at] = t;
+            wait_v[warp][at] = v;
+        }
+        nwait += __popc(m);
+        if (nwait > 28) {
+            __syncwarp();
+            if (lane < nwait) bc_dep_update(wait_v[warp][lane], wait_t[warp][lane], source, sigma, coef, score);
+            __syncwarp();
+            nwait = 0;
         }
     }
+    __syncwarp();
+    if (lane < nwait) bc_dep_update(wait_v[warp][lane], wait_t[warp][lane], source, sigma, coef, score);
 }
 
 // A level runs in the push direction while its frontier's out-edges are fewer than
@@ -349,6 +393,9 @@ struct BcScratch {
     DevBuf fdeg, fpre, fws;  // push levels: frontier out-degrees, their prefix, scan scratch
     std::vector<int64_t> off;  // level L of `order` is [off[L], off[L+1])
     int grid = 1;
+    // the odd levels' coefficients take the place of the push levels' prefix, which the backward sweep
+    // does not need
+    BcPair coefs() const { return BcPair{coef.as<double>(), fpre.as<double>()}; }
     int setup(const tc_graph *g, bool need_score, cudaStream_t s, const tc_part *part = nullptr) {
         if (part) {
             TC_TRY(bpartial.alloc((size_t)(part->R > 0 ? part->R : 1) * 8));
@@ -381,7 +428,7 @@ static int bc_forward_impl(const tc_graph *g, const tc_part *part, int32_t sourc
     double *sigma = w.sigma.as<double>();
     unsigned long long *cnt = w.counter.as<unsigned long long>();  // found vertices, their out-edges
     const int32_t *orp = g->out_rowptr.as<int32_t>();
-    k_bc_init<<<w.grid, BC_THREADS, 0, s>>>(V, source, depth, sigma, w.coef.as<double>(), order);
+    k_bc_init<<<w.grid, BC_THREADS, 0, s>>>(V, source, depth, sigma, order);
     TC_LAUNCH_CHECK();
     w.off.assign(1, 0);
     w.off.push_back(1);
@@ -503,18 +550,22 @@ static int bc_impl(const tc_graph *g, const tc_part *part, const int32_t *source
     double *score = dev_out ? scores_out : w.score.as<double>();
     k_bc_zero<<<w.grid, BC_THREADS, 0, s>>>(V, score);
     TC_LAUNCH_CHECK();
+    const BcPair coef = w.coefs();
     const int32_t small_max = BC_SMALL < g->hub_degree ? BC_SMALL : g->hub_degree;
     for (int32_t k = 0; k < num_sources; ++k) {
         int32_t maxd = 0;
         TC_TRY(bc_forward_impl(g, part, sources[k], w, s, &maxd, nullptr));
+        TC_CUDA(cudaMemsetAsync(coef.even, 0, (size_t)V * 8, s));
+        TC_CUDA(cudaMemsetAsync(coef.odd, 0, (size_t)V * 8, s));
         for (int32_t L = maxd; L >= 0; --L) {
             const int64_t a = w.off[(size_t)L], n = w.off[(size_t)L + 1] - a;
-            const int64_t want4 = (n + 4 * BC_WARPS - 1) / (4 * BC_WARPS);
-            const int grid4 = (int)(want4 < w.grid ? (want4 > 0 ? want4 : 1) : w.grid);
-            k_bc_backward<<<grid4 + g->num_out_hubs, BC_THREADS, 0, s>>>(
+            // one vertex per warp step up to four steps of the whole grid, else four
+            const int32_t per = n <= 4 * (int64_t)w.grid * BC_WARPS ? 1 : 4;
+            const int grid = (int)(n < w.grid ? n : w.grid);
+            k_bc_backward<<<grid + g->num_out_hubs, BC_THREADS, 0, s>>>(
                 g->out_rowptr.as<int32_t>(), g->out_colidx.as<int32_t>(), w.order.as<int32_t>() + a, n,
-                g->out_hubs.as<int32_t>(), g->num_out_hubs, L, sources[k], small_max, g->hub_degree,
-                w.depth.as<int32_t>(), w.sigma.as<double>(), w.coef.as<double>(), score);
+                g->out_hubs.as<int32_t>(), g->num_out_hubs, L, sources[k], small_max, g->hub_degree, per,
+                w.depth.as<int32_t>(), w.sigma.as<double>(), coef.at(L + 1), coef.at(L), score);
             TC_LAUNCH_CHECK();
         }
     }

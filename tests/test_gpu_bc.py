@@ -173,3 +173,19 @@ def test_levels_around_the_warp_queues_flush_sizes(T, n):
         assert np.array_equal(d.cpu().numpy(), wd) and np.array_equal(sg.cpu().numpy(), ws)
     got = T.bc(G, [0, 1]).cpu().numpy()
     np.testing.assert_allclose(got, oracle.bc(g.V, rp, ci, [0, 1]), rtol=1e-12, atol=0)
+
+
+@pytest.mark.parametrize("n", [38911, 38912, 38913, 60001])
+def test_levels_around_the_vertices_per_warp_step(T, n):
+    """A backward level gives a warp one vertex per step up to 38,912 vertices (on 152 SMs), four above,
+    and divides for 32 vertices together.  Two hubs joined by n middle vertices: from one hub each middle
+    vertex lies on one of the n paths to the other, so it scores 1 / n; from a middle vertex the hubs
+    share its paths to the n - 1 others, (n - 1) / 2 each."""
+    g = gg.from_edge_list(n + 2, [(h, 2 + i) for i in range(n) for h in (0, 1)] +
+                          [(2 + i, h) for i in range(n) for h in (0, 1)])
+    G = _load(T, g)
+    got = T.bc(G, [0]).cpu().numpy()
+    assert np.all(got[2:] == 1.0 / n) and np.all(got[:2] == 0.0)
+    got = T.bc(G, [2]).cpu().numpy()
+    np.testing.assert_allclose(got[:2], (n - 1) / 2, rtol=1e-12)  # n additions of 1/2 at most: exact
+    assert np.all(got[2:] == 0.0)
