@@ -145,11 +145,11 @@ typedef struct tc_part_params {
     int32_t smem_stage;       /* pull: 0 = stage each block's contributions in shared
                                  memory whenever W fits (W <= about 41K sources, W % 32 == 0),
                                  -1 = never, 1 = require it (TC_ERR_UNSUPPORTED if W does not fit).
-                                 push: 1 = accumulate each block's destination range in shared
-                                 memory when W * 8 bytes fit (about 29K vertices; the
-                                 TC_BLOCKS_SMEM policy picks that width), 0 / -1 = the global
-                                 scatters.  Measured slower on R-MAT (shared-memory atomics on
-                                 the hub destinations of a range serialise), so not the default */
+                                 push: 1 = require that each block's destination range fits
+                                 shared memory (W * 8 bytes, about 29K vertices; the
+                                 TC_BLOCKS_SMEM policy picks that width) and accumulate FP32
+                                 sums there too; fixed-point sums go through ranges of the
+                                 library's own unless -1 (then always the global scatters) */
     int32_t vertex_order;     /* pull only: TC_ORDER_NATURAL (0) or TC_ORDER_OUTDEGREE (1), below */
     int32_t direct_blocks;    /* renumbered pull only: local rows with a single edge whose source
                                  lies in the first `direct_blocks` blocks leave the blocked CSR

@@ -191,6 +191,48 @@ __device__ __forceinline__ bool grid_sum2_last_cta(double a, double b, double *p
     return true;
 }
 
+// round(y) as a 64-bit two's-complement integer for |y| < 2^62, from the FP32 bits (integer
+// operations only: 64-bit float-to-integer conversions run on the FP64 unit).
+__device__ __forceinline__ unsigned long long fx_round64(float y) {
+    const uint32_t b = __float_as_uint(y);
+    const uint32_t a = b & 0x7fffffffu;
+    const int e = (int)(a >> 23);
+    const unsigned long long m = (a & 0x7fffffu) | (e ? 0x800000u : 0u);
+    const int sh = (e ? e : 1) - 150;  // |y| = m * 2^sh
+    unsigned long long r;
+    if (sh >= 0) r = m << sh;
+    else if (sh <= -25) r = 0ull;
+    else r = (m + (1ull << (-sh - 1))) >> (-sh);  // to nearest, ties away from zero
+    return (b >> 31) ? (0ull - r) : r;
+}
+
+// The dangling mass of a push iteration in fixed point (`scalef` per unit): CTA-wide sum `mine` goes to
+// slot[i]; the last of n arrivals adds the slots and writes D and D / V.  Integers: the same for any
+// division of the vertices among CTAs.  All threads of the CTA call it.
+__device__ __forceinline__ void push_dangling_last(unsigned long long mine, int32_t i, int32_t n,
+                                                   unsigned long long *slot, unsigned *counter, float scalef,
+                                                   double *D, SpreadOut spread) {
+    __shared__ bool am_last4;
+    __shared__ unsigned long long red4[32];
+    if (threadIdx.x == 0) {
+        slot[i] = mine;
+        __threadfence();
+        am_last4 = atomicAdd(counter, 1u) == (unsigned)n - 1u;
+    }
+    __syncthreads();
+    if (!am_last4) return;
+    __threadfence();
+    unsigned long long t = 0;
+    for (int32_t k = threadIdx.x; k < n; k += blockDim.x) t += __ldcg(slot + k);
+    t = block_sum<unsigned long long>(t, red4);
+    if (threadIdx.x == 0) {
+        const double d = (double)(long long)t / (double)scalef;
+        *D = d;
+        spread.write(d);
+        *counter = 0u;
+    }
+}
+
 // Appends to a queue in global memory, staged per warp in shared memory: `count` moves by one atomic
 // per 32 entries (and one per CTA at the end) instead of one per entry or per warp step.  An atomic
 // per entry on one address bounded the traversal levels that had it (BC from 4 sources on a
@@ -246,5 +288,26 @@ struct WarpQueue {
         if (lane < n) queue[wq_base + wq_n[warp] + lane] = buf[lane];
     }
 };
+
+// What the push iteration by destination ranges works on (tc_push.cu); the launch fills W, B and
+// range_count from the partition.
+struct PushCutArgs {
+    float base, damping;          // (1-d)/V and d
+    int drop;                     // 1: dangling mass is not redistributed
+    int32_t V, W, B;              // vertices, width and number of the ranges
+    const float *S_cur;           // D / V of the contributions read
+    double *D_next;               // dangling mass of the ranks written, with D / V in `spread`
+    SpreadOut spread;
+    const float *inv_outdeg;
+    const float *contrib;
+    float *contrib_next;
+    float *rank_out;              // may be null
+    const float *fx_scale;
+    unsigned long long *sums;     // zero between launches; ranges of several tiles meet there
+    int32_t *range_count;
+    unsigned long long *dslot;    // [B]
+    unsigned *counter;
+};
+int launch_push_cut(const tc_part *p, PushCutArgs a, cudaStream_t s);
 
 }  // namespace tc

@@ -228,6 +228,15 @@ struct tc_part {
     tc::DevBuf pperm;           // int32[E]: the loaded CSR position of every partition entry
     tc::DevBuf pvals;           // float[E]: the matrix values in partition order
     int32_t nptiles = 0;        // push, W * 8 bytes within shared memory: tiles of the staged push
+    // push: the edges by destination range of cut_W vertices (fixed-point staged push; tc_push.cu),
+    // built on first use
+    bool cut_tried = false;
+    int32_t smem_stage = 0;     // as asked for: < 0 never staged
+    int32_t cut_W = 0, cut_B = 0, cut_ntiles = 0;
+    tc::DevBuf cut_src;         // int32[E]: source
+    tc::DevBuf cut_dst;         // uint16[E]: destination minus its range's first vertex
+    tc::DevBuf cut_tiles;       // int4[cut_ntiles]: (range, first edge, end edge, tiles of the range)
+    tc::DevBuf cut_count;       // int32[cut_B]: finished tiles of a range that has several (zero between launches)
     tc::DevBuf ptiles;          // int4[nptiles]: (block, first edge low 31 bits, high bits, edges)
     // ---- shared-memory staged format (pull, W <= smem capacity; see tc_tile.cu) ----
     bool tiled = false;
@@ -270,6 +279,7 @@ int32_t tile_max_width(int max_smem_optin);
 // Staged push (tc_push.cu): widest destination range in shared memory, its tiles, the scatter.
 int32_t push_smem_width(int max_smem_optin);
 int build_push_tiles(tc_part *p, int sms, cudaStream_t s);
+int ensure_push_cut(tc_part *p, cudaStream_t s);
 int launch_push_smem(const tc_part *p, const float *contrib, void *sums, const float *fx_scale, bool fixed,
                      cudaStream_t s);
 int build_tiles(tc_part *p, int sms, cudaStream_t s);

@@ -708,21 +708,6 @@ __global__ void __launch_bounds__(PR_THREADS) k_pr_init(const float *__restrict_
 // form, order-dependent rounding).
 // ---------------------------------------------------------------------------------------------
 
-// round(y) as a 64-bit two's-complement integer for |y| < 2^62, from the FP32 bits (integer
-// operations only: 64-bit float-to-integer conversions run on the FP64 unit).
-__device__ __forceinline__ unsigned long long fx_round64(float y) {
-    const uint32_t b = __float_as_uint(y);
-    const uint32_t a = b & 0x7fffffffu;
-    const int e = (int)(a >> 23);
-    const unsigned long long m = (a & 0x7fffffu) | (e ? 0x800000u : 0u);
-    const int sh = (e ? e : 1) - 150;  // |y| = m * 2^sh
-    unsigned long long r;
-    if (sh >= 0) r = m << sh;
-    else if (sh <= -25) r = 0ull;
-    else r = (m + (1ull << (-sh - 1))) >> (-sh);  // to nearest, ties away from zero
-    return (b >> 31) ? (0ull - r) : r;
-}
-
 template <bool FIXED>
 __device__ __forceinline__ void push_add(void *sums, int32_t d, float c, float scalef) {
     if (FIXED) atomicAdd(static_cast<unsigned long long *>(sums) + d, fx_round64(c * scalef));
@@ -818,6 +803,8 @@ __global__ void __launch_bounds__(PR_THREADS) k_push_edges(const int32_t *__rest
 template <bool FIXED>
 __global__ void __launch_bounds__(PR_THREADS) k_push_update(void *sums, UpdateArgs u) {
     __shared__ float fred[32];
+    __shared__ unsigned long long ured[32];
+    unsigned long long dfix = 0;  // FIXED: the dangling mass in the sums' fixed point, exact in any order
     const float spread = spread_of(u);
     const float inv_scalef = FIXED ? 1.0f / push_scale(u.fx_scale) : 1.0f;  // a power of two
     float dsum = 0.0f;
@@ -835,7 +822,15 @@ __global__ void __launch_bounds__(PR_THREADS) k_push_update(void *sums, UpdateAr
             s = *sp;
             *sp = 0.0f;
         }
-        dsum += apply_update(u, (int32_t)v, s, spread);
+        const float d = apply_update(u, (int32_t)v, s, spread);
+        if (FIXED) dfix += fx_round64(d * push_scale(u.fx_scale));
+        else dsum += d;
+    }
+    if (FIXED) {
+        dfix = block_sum<unsigned long long>(dfix, ured);
+        push_dangling_last(dfix, blockIdx.x, gridDim.x, reinterpret_cast<unsigned long long *>(u.dpart), u.counter,
+                           push_scale(u.fx_scale), u.D_next, spread_out(u));
+        return;
     }
     const float bs = block_sum<float>(dsum, fred);
     grid_sum_last_cta((double)bs, u.dpart, u.counter, u.D_next, 0.0, spread_out(u));
@@ -1028,17 +1023,21 @@ static int pagerank_impl(const tc_graph *cg, const tc_part *part, const tc_pr_pa
     if (max_ctas_hint > max_ctas) max_ctas = max_ctas_hint;
     if (g_upd > max_ctas) max_ctas = g_upd;
     if (g_merge > max_ctas) max_ctas = g_merge;
+    // push: fixed-point sums unless FP32 atomics are asked for; unless a TWC warp threshold (lb_warp_min
+    // or a per-block table) is given, a partition's scatter goes by destination ranges, else edge-parallel
+    const bool push_fixed = pp->merge_mode != TC_PUSH_FLOAT;
+    const bool push_whole = push && pp->lb_warp_min == 0 && !(part && part->lb_tab.p);  // no TWC threshold
+    if (push_whole && part && push_fixed) TC_TRY(ensure_push_cut(const_cast<tc_part *>(part), s));
+    const bool push_cut = push_whole && part && push_fixed && part->cut_ntiles > 0;
+    if (push_cut && part->cut_B > max_ctas) max_ctas = part->cut_B;  // one dangling slot per range
     if (part && !push && part->nranges > max_ctas) max_ctas = part->nranges;  // one dangling slot per range
 
     PrState st;
     TC_TRY(prepare_state(g, pp, ranks_out, push, max_ctas, &st));
     TC_CUDA(cudaMemsetAsync(st.counter, 0, 16, s));  // counter, merge work queue and the error flag
     if (push) TC_CUDA(cudaMemsetAsync(st.sums, 0, (size_t)V * 8, s));
-    // push: fixed-point sums unless FP32 atomics are asked for; the edge-parallel scatter unless
-    // a TWC warp threshold (lb_warp_min or a per-block table) is given
-    const bool push_fixed = pp->merge_mode != TC_PUSH_FLOAT;
-    const bool push_staged = push && part && part->nptiles > 0 && pp->lb_warp_min == 0 && !part->lb_tab.p;
-    const bool push_edges = push && !push_staged && pp->lb_warp_min == 0 && !(part && part->lb_tab.p);
+    const bool push_staged = push_whole && !push_cut && part && part->nptiles > 0;
+    const bool push_edges = push_whole && !push_cut && !push_staged;
     const int32_t *esrc = nullptr;
     int64_t nedges = 0;
     int g_edges = 1;
@@ -1113,13 +1112,14 @@ static int pagerank_impl(const tc_graph *cg, const tc_part *part, const tc_pr_pa
     }
     for (int it = 0; it < pp->iters; ++it) {
         const bool last = it == pp->iters - 1;
-        const float *cur = push ? st.contrib[0] : st.contrib[it & 1];
+        const bool in_place = push && !push_cut;
+        const float *cur = in_place ? st.contrib[0] : st.contrib[it & 1];
         u.D_cur = st.D + (it & 1);
         u.D_next = st.D + ((it + 1) & 1);
         u.S_cur = st.S + (it & 1);
         u.S_next = st.S + ((it + 1) & 1);
         u.rank_out = last ? st.rank_dev : nullptr;
-        u.contrib_next = push ? st.contrib[0] : st.contrib[(it + 1) & 1];
+        u.contrib_next = in_place ? st.contrib[0] : st.contrib[(it + 1) & 1];
         u.cur = cur;
         Timer t1;
         TC_TRY(t1.begin(pp->profile != 0, s, &ms_gather));
@@ -1129,7 +1129,26 @@ static int pagerank_impl(const tc_graph *cg, const tc_part *part, const tc_pr_pa
         lb.blk_rows = part ? part->blk_rows_dev.as<int64_t>() : nullptr;
         lb.B = part ? part->B : 1;
         if (push) {
-            if (push_staged)
+            if (push_cut) {
+                PushCutArgs a = {};
+                a.base = u.base;
+                a.damping = u.damping;
+                a.drop = u.drop;
+                a.V = V;
+                a.S_cur = u.S_cur;
+                a.D_next = u.D_next;
+                a.spread.out = u.S_next;
+                a.spread.V = V;
+                a.inv_outdeg = u.inv_outdeg;
+                a.contrib = cur;
+                a.contrib_next = u.contrib_next;
+                a.rank_out = u.rank_out;
+                a.fx_scale = st.scale;
+                a.sums = reinterpret_cast<unsigned long long *>(st.sums);
+                a.dslot = reinterpret_cast<unsigned long long *>(st.dpart);
+                a.counter = st.counter;
+                TC_TRY(launch_push_cut(part, a, s));
+            } else if (push_staged)
                 TC_TRY(launch_push_smem(part, cur, st.sums, st.scale, push_fixed, s));
             else if (push_edges && push_fixed)
                 k_push_edges<true><<<g_edges, PR_THREADS, 0, s>>>(esrc, ci, nedges, cur, st.sums, st.scale);
@@ -1172,7 +1191,7 @@ static int pagerank_impl(const tc_graph *cg, const tc_part *part, const tc_pr_pa
         TC_LAUNCH_CHECK();
         ++launches;
         TC_TRY(t1.end());
-        if (push || part) {
+        if ((push || part) && !push_cut) {  // (the cut's scatter has updated the ranks)
             Timer t2;
             TC_TRY(t2.begin(pp->profile != 0, s, &ms_merge));
             if (push) {

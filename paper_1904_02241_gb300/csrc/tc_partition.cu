@@ -499,6 +499,7 @@ static int partition_impl(const tc_graph *g, int dir, int32_t num_blocks, const 
     const int32_t *ci = dir == TC_PULL ? g->in_colidx.as<int32_t>() : g->out_colidx.as<int32_t>();
     p->g = g;
     p->dir = dir;
+    p->smem_stage = pp ? pp->smem_stage : 0;
     p->V = V;
     p->E = E;
     const int order = pp ? pp->vertex_order : TC_ORDER_NATURAL;

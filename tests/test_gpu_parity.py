@@ -827,3 +827,26 @@ def test_bfs_blocked_levels_from_shared_memory(T, name, B):
         lv, st = T.bfs_pull(G, P, s, tocab_threshold=0.0, return_stats=True)
         np.testing.assert_array_equal(lv.cpu().numpy(), oracle.bfs(g.V, rp, ci, s))
         assert st.tocab_levels == st.levels
+
+
+@pytest.mark.parametrize("V", [1, 31, 33, 9120, 9121, 70001])
+@pytest.mark.parametrize("hub", [False, True])
+def test_push_destination_ranges_give_the_scatters_bits(T, V, hub):
+    """The fixed-point push by destination ranges (285 of 32 vertices at V = 9,120) against the row
+    scatter, which takes the edges in another order: the same integer sums, so the same bits, with ranks
+    of either sign, ranges without edges, and a range of several tiles (half the edges into one vertex)."""
+    rng = np.random.default_rng(V)
+    m = 12 * V
+    e = np.stack([rng.integers(0, V, m), rng.integers(0, (V + 1) // 2, m)], axis=1)
+    if hub:
+        e[: m // 2, 1] = V // 3
+    g = gg.from_edge_list(V, e)
+    G = _load(T, g)
+    init = torch.tensor(rng.standard_normal(V) / V, dtype=torch.float32).cuda()
+    for B in (1, min(3, V)):
+        P = T.tocab_partition(G, T.TC_PUSH, B)
+        for kw in ({}, {"init": init}, {"dangling": "drop"}):
+            a = T.pagerank_push(G, P, iters=4, **kw).cpu()
+            assert torch.equal(a, T.pagerank_push(G, P, iters=4, **kw).cpu())
+            assert torch.equal(a, T.pagerank_push(G, P, iters=4, lb_warp_min=8, **kw).cpu())
+            assert torch.equal(a, T.pagerank_push(G, None, iters=4, **kw).cpu())
