@@ -206,32 +206,52 @@ __device__ __forceinline__ unsigned long long fx_round64(float y) {
     return (b >> 31) ? (0ull - r) : r;
 }
 
-// The dangling mass of a push iteration in fixed point (`scalef` per unit): CTA-wide sum `mine` goes to
-// slot[i]; the last of n arrivals adds the slots and writes D and D / V.  Integers: the same for any
-// division of the vertices among CTAs.  All threads of the CTA call it.
-__device__ __forceinline__ void push_dangling_last(unsigned long long mine, int32_t i, int32_t n,
-                                                   unsigned long long *slot, unsigned *counter, float scalef,
-                                                   double *D, SpreadOut spread) {
-    __shared__ bool am_last4;
-    __shared__ unsigned long long red4[32];
-    if (threadIdx.x == 0) {
-        slot[i] = mine;
-        __threadfence();
-        am_last4 = atomicAdd(counter, 1u) == (unsigned)n - 1u;
-    }
-    __syncthreads();
-    if (!am_last4) return;
-    __threadfence();
+// The dangling mass of a push iteration in fixed point (`scalef` per unit).  A thread adds its vertices to
+// a DanglingSum; all threads of the CTA call finish(i): the CTA's sum goes to slot[i], and the last of n
+// arrivals adds the slots and writes D and D / V.  Integers: the same for any division of the vertices
+// among CTAs.  Ranks that are not finite (from initial ranks that are not) make D so too: they are added
+// as FP32 beside the sum, and their sum takes the slot, marked in bits that no sum of finite ranks
+// (below 2^56) has.
+struct DanglingSum {
+    static constexpr unsigned long long MARK = 0x4000000000000000ull;
     unsigned long long t = 0;
-    for (int32_t k = threadIdx.x; k < n; k += blockDim.x) t += __ldcg(slot + k);
-    t = block_sum<unsigned long long>(t, red4);
-    if (threadIdx.x == 0) {
-        const double d = (double)(long long)t / (double)scalef;
-        *D = d;
-        spread.write(d);
-        *counter = 0u;
+    float odd = 0.0f;  // sum of the ranks that are not finite
+    __device__ __forceinline__ void add(float r, float scalef) {
+        if (fabsf(r) <= 3.402823466e38f) t += fx_round64(r * scalef);
+        else odd += r;
     }
-}
+    __device__ __forceinline__ void finish(int32_t i, int32_t n, unsigned long long *slot, unsigned *counter,
+                                           float scalef, double *D, SpreadOut spread) {
+        __shared__ bool am_last4;
+        __shared__ unsigned long long red4[32];
+        __shared__ float redf4[32];
+        t = block_sum<unsigned long long>(t, red4);
+        if (__syncthreads_or(odd != 0.0f)) t = MARK | __float_as_uint(block_sum<float>(odd, redf4));
+        if (threadIdx.x == 0) {
+            slot[i] = t;
+            __threadfence();
+            am_last4 = atomicAdd(counter, 1u) == (unsigned)n - 1u;
+        }
+        __syncthreads();
+        if (!am_last4) return;
+        __threadfence();
+        t = 0;
+        odd = 0.0f;
+        for (int32_t k = threadIdx.x; k < n; k += blockDim.x) {
+            const unsigned long long x = __ldcg(slot + k);
+            if ((x >> 56) == (MARK >> 56)) odd += __uint_as_float((uint32_t)x);
+            else t += x;
+        }
+        t = block_sum<unsigned long long>(t, red4);
+        odd = block_sum<float>(odd, redf4);
+        if (threadIdx.x == 0) {
+            const double d = (double)(long long)t / (double)scalef + (double)odd;
+            *D = d;
+            spread.write(d);
+            *counter = 0u;
+        }
+    }
+};
 
 // Appends to a queue in global memory, staged per warp in shared memory: `count` moves by one atomic
 // per 32 entries (and one per CTA at the end) instead of one per entry or per warp step.  An atomic

@@ -803,8 +803,7 @@ __global__ void __launch_bounds__(PR_THREADS) k_push_edges(const int32_t *__rest
 template <bool FIXED>
 __global__ void __launch_bounds__(PR_THREADS) k_push_update(void *sums, UpdateArgs u) {
     __shared__ float fred[32];
-    __shared__ unsigned long long ured[32];
-    unsigned long long dfix = 0;  // FIXED: the dangling mass in the sums' fixed point, exact in any order
+    DanglingSum dfix;  // FIXED: the dangling mass in the sums' fixed point, exact in any order
     const float spread = spread_of(u);
     const float inv_scalef = FIXED ? 1.0f / push_scale(u.fx_scale) : 1.0f;  // a power of two
     float dsum = 0.0f;
@@ -823,13 +822,12 @@ __global__ void __launch_bounds__(PR_THREADS) k_push_update(void *sums, UpdateAr
             *sp = 0.0f;
         }
         const float d = apply_update(u, (int32_t)v, s, spread);
-        if (FIXED) dfix += fx_round64(d * push_scale(u.fx_scale));
+        if (FIXED) dfix.add(d, push_scale(u.fx_scale));
         else dsum += d;
     }
     if (FIXED) {
-        dfix = block_sum<unsigned long long>(dfix, ured);
-        push_dangling_last(dfix, blockIdx.x, gridDim.x, reinterpret_cast<unsigned long long *>(u.dpart), u.counter,
-                           push_scale(u.fx_scale), u.D_next, spread_out(u));
+        dfix.finish(blockIdx.x, gridDim.x, reinterpret_cast<unsigned long long *>(u.dpart), u.counter,
+                    push_scale(u.fx_scale), u.D_next, spread_out(u));
         return;
     }
     const float bs = block_sum<float>(dsum, fred);

@@ -197,7 +197,6 @@ __global__ void __launch_bounds__(PS_THREADS, 2) k_push_cut(const int4 *__restri
     extern __shared__ __align__(16) unsigned char psm[];
     uint32_t *acc_lo = reinterpret_cast<uint32_t *>(psm);
     uint32_t *acc_hi = acc_lo + a.W;
-    __shared__ unsigned long long red[32];
     __shared__ bool s_last;
     const int4 t = tiles[blockIdx.x];  // (range, first edge, end edge, tiles of the range)
     const int32_t lo = t.x * a.W;
@@ -247,7 +246,7 @@ __global__ void __launch_bounds__(PS_THREADS, 2) k_push_cut(const int4 *__restri
     }
     const float spread = a.drop ? 0.0f : *a.S_cur;
     const float inv_scalef = 1.0f / scalef;  // a power of two
-    unsigned long long dsum = 0;
+    DanglingSum dangling;
     for (int32_t v = threadIdx.x; v < w; v += PS_THREADS) {
         unsigned long long x;
         if (shared_range) {
@@ -260,10 +259,9 @@ __global__ void __launch_bounds__(PS_THREADS, 2) k_push_cut(const int4 *__restri
         if (a.rank_out) a.rank_out[lo + v] = r;
         const float inv = __ldg(a.inv_outdeg + lo + v);
         a.contrib_next[lo + v] = r * inv;
-        if (inv == 0.0f) dsum += fx_round64(r * scalef);
+        if (inv == 0.0f) dangling.add(r, scalef);
     }
-    dsum = block_sum<unsigned long long>(dsum, red);
-    push_dangling_last(dsum, t.x, a.B, a.dslot, a.counter, scalef, a.D_next, a.spread);
+    dangling.finish(t.x, a.B, a.dslot, a.counter, scalef, a.D_next, a.spread);
 }
 
 // First edge of every range (keys ascending by range, n of them), b in [0, B].

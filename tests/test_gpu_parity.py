@@ -850,3 +850,17 @@ def test_push_destination_ranges_give_the_scatters_bits(T, V, hub):
             assert torch.equal(a, T.pagerank_push(G, P, iters=4, **kw).cpu())
             assert torch.equal(a, T.pagerank_push(G, P, iters=4, lb_warp_min=8, **kw).cpu())
             assert torch.equal(a, T.pagerank_push(G, None, iters=4, **kw).cpu())
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_push_dangling_mass_that_is_not_finite(T, bad):
+    """A dangling vertex whose initial rank is not finite leaves no finite rank on any fixed-point push
+    path, however many iterations follow (its mass goes to every vertex)."""
+    g = gg.from_edge_list(5000, [(i, (7 * i + k) % 5000) for i in range(4000) for k in (1, 2, 5)])
+    G = _load(T, g)
+    init = torch.full((g.V,), 1.0 / g.V)
+    init[4500] = bad
+    for P, lb in ((T.tocab_partition(G, T.TC_PUSH, 2), 0), (None, 0), (None, 8)):
+        for iters in (1, 2, 5):
+            r = T.pagerank_push(G, P, iters=iters, init=init.cuda(), lb_warp_min=lb)
+            assert not torch.isfinite(r).any()
