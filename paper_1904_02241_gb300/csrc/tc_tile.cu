@@ -377,6 +377,10 @@ __global__ void k_tile_wtab(const int32_t *rowptr, const int64_t *cum, const int
     }
 }
 
+// A tile costs some 4 us besides its rows (its launch, the copy of the block's values, its first and last
+// chunks), 100,000 units of the row costs.  Up to 2.5 times that per tile another wave does not pay.
+constexpr int64_t TILE_SMALL = 250000;
+
 int build_tiles(tc_part *p, int sms, cudaStream_t s) {
     p->tiled = false;
     const int64_t R = p->R;
@@ -410,8 +414,13 @@ int build_tiles(tc_part *p, int sms, cudaStream_t s) {
     TC_TRY(p->heads.alloc((size_t)(npad + WCH) / 8 + 64));
     TC_CUDA(cudaMemsetAsync(p->col16.p, 0, (size_t)(npad + WCH) * 2, s));
     TC_CUDA(cudaMemsetAsync(p->heads.p, 0, (size_t)(npad + WCH) / 8 + 64, s));
-    // tiles: the rows of every block with edges are cut into n_b = max(1, round(cost_b / T)) tiles
-    // of equal estimated cost, T = the total over three waves of one CTA per SM
+    // tiles: the rows of every block with edges are cut into n_b = max(1, round(cost_b / T)) tiles of
+    // equal estimated cost, T = the total over whole waves of one CTA per SM:
+    //   * three waves where blocks are uneven (the largest-first order then evens out what the estimate
+    //     misses: R-MAT 24 renumbered, 254 us per gather against 278 us with two and 355 us with one);
+    //   * the block count's own waves where the blocks are even (6M uniform: 113 us against 125 us);
+    //   * one wave where a tile costs little next to TILE_SMALL (R-MAT 16: 10 us against 19 us, R-MAT 20
+    //     renumbered: 32 us against 35 us).
     DevBuf wrow, cum, cw;
     TC_TRY(wrow.alloc(((size_t)R + 1) * 4));
     TC_TRY(cum.alloc(((size_t)R + 1) * 8));
@@ -426,14 +435,27 @@ int build_tiles(tc_part *p, int sms, cudaStream_t s) {
     std::vector<int64_t> h_cw((size_t)B + 1);
     TC_CUDA(cudaMemcpyAsync(h_cw.data(), cw.p, ((size_t)B + 1) * 8, cudaMemcpyDeviceToHost, s));
     TC_CUDA(cudaStreamSynchronize(s));
-    const int64_t T = h_cw[B] / (3LL * sms) > 0 ? h_cw[B] / (3LL * sms) : 1;
-    std::vector<int4> h_tiles;
+    int64_t maxb = 0, nblk = 0;
     for (int32_t b = 0; b < B; ++b) {
-        if (p->h_blk_edges[b + 1] == p->h_blk_edges[b]) continue;
-        int64_t n = (h_cw[b + 1] - h_cw[b] + T / 2) / T;
-        if (n < 1) n = 1;
-        if (n > p->h_blk_rows[b + 1] - p->h_blk_rows[b]) n = p->h_blk_rows[b + 1] - p->h_blk_rows[b];
-        for (int64_t k = 0; k < n; ++k) h_tiles.push_back(make_int4(b, (int)k, (int)n, 0));
+        maxb = std::max(maxb, h_cw[b + 1] - h_cw[b]);
+        nblk += h_cw[b + 1] > h_cw[b];
+    }
+    int64_t waves = 3;
+    if (h_cw[B] < 3 * sms * TILE_SMALL) waves = 1;
+    else if (nblk % sms == 0 && maxb * nblk < h_cw[B] * 9 / 8) waves = nblk / sms;
+    int64_t T = h_cw[B] / (waves * sms) > 0 ? h_cw[B] / (waves * sms) : 1;
+    std::vector<int4> h_tiles;
+    for (;; T += T / 64 + 1) {
+        h_tiles.clear();
+        for (int32_t b = 0; b < B; ++b) {
+            if (p->h_blk_edges[b + 1] == p->h_blk_edges[b]) continue;
+            int64_t n = (h_cw[b + 1] - h_cw[b] + T / 2) / T;
+            if (n < 1) n = 1;
+            if (n > p->h_blk_rows[b + 1] - p->h_blk_rows[b]) n = p->h_blk_rows[b + 1] - p->h_blk_rows[b];
+            for (int64_t k = 0; k < n; ++k) h_tiles.push_back(make_int4(b, (int)k, (int)n, 0));
+        }
+        // a single wave must not spill into a second one for the rounding of the blocks' tile counts
+        if (waves > 1 || nblk > sms || (int64_t)h_tiles.size() <= sms) break;
     }
     const int64_t ntiles = (int64_t)h_tiles.size();
     if (ntiles * (TWARPS + 1) > INT32_MAX) return fail(TC_ERR_UNSUPPORTED, "build_tiles: too many tiles");

@@ -864,3 +864,21 @@ def test_push_dangling_mass_that_is_not_finite(T, bad):
         for iters in (1, 2, 5):
             r = T.pagerank_push(G, P, iters=iters, init=init.cuda(), lb_warp_min=lb)
             assert not torch.isfinite(r).any()
+
+
+@pytest.mark.parametrize("V,B", [(65536, 4), (65536, 13), (70001, 200), (20000, 1)])
+def test_gather_tiles_of_small_graphs_fit_one_wave(T, V, B):
+    """Small graphs get one wave of tiles: at most as many as there are SMs, whatever the rounding of the
+    blocks' shares, unless the blocks alone are more; a block with most of the edges is still cut."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rng = np.random.default_rng(B)
+    m = 12 * V
+    src = rng.integers(0, V, m)
+    src[: m // 2] %= max(1, V // (2 * B))  # half the edges from the first block
+    g = gg.from_edge_list(V, np.stack([src, rng.integers(0, V, m)], axis=1))
+    G = _load(T, g)
+    P = T.tocab_partition(G, T.TC_PULL, B)
+    assert P.num_tiles <= sms if P.num_blocks <= sms else P.num_tiles < 2 * P.num_blocks
+    if 1 < P.num_blocks < sms:
+        assert P.num_tiles > sms // 2
+    assert l1_rel(T.pagerank_pull(G, P).cpu().numpy(), _oracle_pr(g)) <= TOL
