@@ -882,3 +882,20 @@ def test_gather_tiles_of_small_graphs_fit_one_wave(T, V, B):
     if 1 < P.num_blocks < sms:
         assert P.num_tiles > sms // 2
     assert l1_rel(T.pagerank_pull(G, P).cpu().numpy(), _oracle_pr(g)) <= TOL
+
+
+@pytest.mark.parametrize("order", ["natural", "outdegree"])
+def test_partition_of_rows_with_long_gaps(T, order):
+    """Rows found from edge positions: chunks of edges that start inside a long row, rows of one edge, and
+    runs of many thousand empty rows between them."""
+    V = 300007
+    rng = np.random.default_rng(9)
+    near = np.concatenate([np.arange(40), 100000 + np.arange(3000), V - 1 - np.arange(5)])
+    e = np.concatenate([np.stack([rng.integers(0, V, 9000), np.full(9000, 7)], axis=1),      # long rows of G^T
+                        np.stack([rng.integers(0, V, 5000), np.full(5000, V - 1)], axis=1),
+                        np.stack([rng.choice(near, 20000), rng.choice(near, 20000)], axis=1)])
+    g = gg.from_edge_list(V, e)
+    G = _load(T, g)
+    P = T.tocab_partition(G, T.TC_PULL, 3 if order == "natural" else 0, block_policy="smem", order=order)
+    assert l1_rel(T.pagerank_pull(G, P).cpu().numpy(), _oracle_pr(g)) <= TOL
+    assert l1_rel(T.pagerank_push(G, T.tocab_partition(G, T.TC_PUSH, 2)).cpu().numpy(), _oracle_pr(g)) <= TOL
