@@ -12,31 +12,57 @@ namespace tc {
 constexpr int BFS_THREADS = 256;
 constexpr int BFS_WARPS = BFS_THREADS / 32;
 
-__device__ __forceinline__ bool in_front(const uint32_t *__restrict__ front, int32_t u) {
-    return (__ldg(front + (u >> 5)) >> (u & 31)) & 1u;
-}
+// Where a scan looks a source up: the frontier bitmap, or a slice of it in shared memory that starts at
+// source lo (a multiple of 32).
+struct FrontBits {
+    const uint32_t *__restrict__ front;
+    __device__ __forceinline__ uint32_t word(int32_t u) const { return __ldg(front + (u >> 5)); }
+};
+struct SliceBits {
+    const uint32_t *sl;
+    int32_t lo;
+    __device__ __forceinline__ uint32_t word(int32_t u) const { return sl[(u - lo) >> 5]; }
+};
 
-// Does row [s, e) hold a source in the frontier?  Lane-serial scan with early exit.
-__device__ __forceinline__ bool scan_serial(const int32_t *__restrict__ colidx, int32_t s, int32_t e,
-                                            const uint32_t *__restrict__ front) {
-    for (int32_t i = s; i < e; ++i)
-        if (in_front(front, __ldg(colidx + i))) return true;
+// Does one of the lane's edges [s, e) come from the frontier?  Early exit after 1, 4, 8, 12, ... edges: the
+// loads of a step are in flight together (one by one, a row is a chain of two dependent round trips per
+// edge), and the first edge alone, which is a hit for most rows when the frontier is large.
+template <int N, class Bits>
+__device__ __forceinline__ bool scan_step(const int32_t *__restrict__ colidx, int32_t i, int32_t e, Bits bits) {
+    int32_t c[N];
+    uint32_t hit = 0;
+#pragma unroll
+    for (int k = 0; k < N; ++k) c[k] = k < e - i ? __ldg(colidx + i + k) : -1;
+#pragma unroll
+    for (int k = 0; k < N; ++k) hit |= (c[k] >= 0 ? bits.word(c[k]) : 0u) >> (c[k] & 31);
+    return hit & 1u;
+}
+template <class Bits>
+__device__ __forceinline__ bool scan_serial(const int32_t *__restrict__ colidx, int32_t s, int32_t e, Bits bits) {
+    if (s >= e) return false;
+    if (scan_step<1>(colidx, s, e, bits)) return true;
+    if (e - s > 1 && scan_step<3>(colidx, s + 1, e, bits)) return true;
+    for (int32_t left = e - s - 4; left > 0; left -= 4)
+        if (scan_step<4>(colidx, e - left, e, bits)) return true;
     return false;
 }
 
-// Warp-cooperative scan of the rows flagged in `wm` (one at a time, early exit per chunk).
+// Warp-cooperative scan of the rows flagged in `wm` (one at a time, early exit per chunk of 64 edges).
+template <class Bits>
 __device__ __forceinline__ bool scan_warp_rows(unsigned wm, int32_t s, int32_t e, const int32_t *__restrict__ colidx,
-                                               const uint32_t *__restrict__ front, bool found) {
+                                               Bits bits, bool found) {
     const int lane = threadIdx.x & 31;
     while (wm) {
         const int l = __ffs(wm) - 1;
         wm &= wm - 1;
         const int32_t ws = __shfl_sync(0xffffffffu, s, l), we = __shfl_sync(0xffffffffu, e, l);
         bool hit = false;
-        for (int32_t base = ws; base < we; base += 32) {
-            const int32_t i = base + lane;
-            const bool h = i < we && in_front(front, __ldg(colidx + i));
-            if (__any_sync(0xffffffffu, h)) {
+        for (int64_t base = ws; base < we; base += 64) {
+            const int64_t i = base + lane;
+            const int32_t c0 = i < we ? __ldg(colidx + i) : -1, c1 = i + 32 < we ? __ldg(colidx + i + 32) : -1;
+            const uint32_t h0 = (c0 >= 0 ? bits.word(c0) : 0u) >> (c0 & 31);
+            const uint32_t h1 = (c1 >= 0 ? bits.word(c1) : 0u) >> (c1 & 31);
+            if (__any_sync(0xffffffffu, (h0 | h1) & 1u)) {
                 hit = true;
                 break;
             }
@@ -44,6 +70,20 @@ __device__ __forceinline__ bool scan_warp_rows(unsigned wm, int32_t s, int32_t e
         if (lane == l) found = hit;
     }
     return found;
+}
+
+// The rows of a warp's candidates, a lane each: short rows whole, the first SCAN_PROBE edges of a longer
+// one; the longer rows without a hit there go to the whole warp one after the other, which is what a
+// level waits for (the first pull level of a search on a symmetrised R-MAT 22: 93 us with every long row
+// going there and one edge at a time, 49 us so).
+constexpr int SCAN_PROBE = 16;
+template <class Bits>
+__device__ __forceinline__ bool scan_rows(bool cand, int32_t s, int32_t e, const int32_t *__restrict__ colidx,
+                                          Bits bits) {
+    const bool is_long = e - s >= 32;
+    const bool found = cand && scan_serial(colidx, s, is_long ? s + SCAN_PROBE : e, bits);
+    return scan_warp_rows(__ballot_sync(0xffffffffu, cand && is_long && !found), is_long ? s + SCAN_PROBE : s, e, colidx,
+                          bits, found);
 }
 
 __global__ void __launch_bounds__(BFS_THREADS) k_bfs_init(int32_t *level, uint32_t *visited, uint32_t *front,
@@ -59,7 +99,7 @@ __global__ void __launch_bounds__(BFS_THREADS) k_bfs_init(int32_t *level, uint32
 
 // Unblocked pull level.  next is written whole (one word per warp), visited updated,
 // count accumulates the size of the new frontier.
-__global__ void __launch_bounds__(BFS_THREADS) k_bfs_pull_level(const int32_t *__restrict__ rowptr,
+__global__ void __launch_bounds__(BFS_THREADS, 8) k_bfs_pull_level(const int32_t *__restrict__ rowptr,
                                                                 const int32_t *__restrict__ colidx, int32_t V,
                                                                 int32_t nwords, const uint32_t *__restrict__ front,
                                                                 uint32_t *__restrict__ next, uint32_t *visited,
@@ -81,10 +121,7 @@ __global__ void __launch_bounds__(BFS_THREADS) k_bfs_pull_level(const int32_t *_
                 s = __ldg(rowptr + v);
                 e = __ldg(rowptr + v + 1);
             }
-            const int32_t deg = e - s;
-            bool found = false;
-            if (cand && deg < 32) found = scan_serial(colidx, s, e, front);
-            found = scan_warp_rows(__ballot_sync(0xffffffffu, cand && deg >= 32), s, e, colidx, front, found);
+            const bool found = scan_rows(cand, s, e, colidx, FrontBits{front});
             nb = __ballot_sync(0xffffffffu, found);
             if (found) {
                 level[v] = new_level;
@@ -106,7 +143,7 @@ __global__ void __launch_bounds__(BFS_THREADS) k_bfs_pull_level(const int32_t *_
 // TOCAB level, phase 1 (Alg. 4 form for traversal): local row r of the row space belongs to
 // destination id_map[r]; bit r of rowbits = "some in-edge of r inside its block comes from
 // the frontier", computed only for unvisited destinations.
-__global__ void __launch_bounds__(BFS_THREADS) k_bfs_block_level(const int32_t *__restrict__ rowptr,
+__global__ void __launch_bounds__(BFS_THREADS, 8) k_bfs_block_level(const int32_t *__restrict__ rowptr,
                                                                  const int32_t *__restrict__ colidx,
                                                                  const int32_t *__restrict__ id_map, int64_t R,
                                                                  const uint32_t *__restrict__ front,
@@ -127,10 +164,7 @@ __global__ void __launch_bounds__(BFS_THREADS) k_bfs_block_level(const int32_t *
                 e = __ldg(rowptr + r + 1);
             }
         }
-        const int32_t deg = e - s;
-        bool found = false;
-        if (cand && deg < 32) found = scan_serial(colidx, s, e, front);
-        found = scan_warp_rows(__ballot_sync(0xffffffffu, cand && deg >= 32), s, e, colidx, front, found);
+        const bool found = scan_rows(cand, s, e, colidx, FrontBits{front});
         const uint32_t nb = __ballot_sync(0xffffffffu, found);
         if (lane == 0) rowbits[grp] = nb;
     }
@@ -143,7 +177,9 @@ __global__ void __launch_bounds__(BFS_THREADS) k_bfs_block_level(const int32_t *
 //   stream : the group's edges are read as one coalesced stream and every edge is tested; the row of
 //            a hit comes from one ballot over the row offsets.  For small frontiers, where nearly every
 //            edge is scanned anyway;
-//   else   : a lane per row (a warp per row from 32 edges) with early exit at the first hit.
+//   else   : a lane per row with early exit (scan_rows).  Streaming here too, with an edge's row from the
+//            count of rows started up to it, was bound by its instructions: 385 against 363 us on the
+//            level with the largest frontier with cold caches, and slower still with warm ones.
 // Bound by reading the edges when it streams; k_bfs_block_level walks a row per lane there and waits
 // on one uncoalesced load and one random bitmap read at a time.  Two searches on a symmetrised R-MAT of
 // 5M vertices, 8 blocks, every level blocked: 5,781 us with that kernel alone (1,018 us for each of the
@@ -196,19 +232,28 @@ __global__ void __launch_bounds__(BLK_THREADS, 2) k_bfs_block_smem(
             empty = !__syncthreads_or(any != 0u);
             held = b;
         }
+        // the next group's row offsets and vertices load while this one is scanned
+        int32_t nv = -1, ns = INT32_MAX, ne = 0;
+        auto rows_of = [&](int64_t r) {
+            nv = -1;
+            ns = INT32_MAX;
+            ne = 0;
+            if (r < c1) {
+                nv = __ldg(id_map + r);
+                ns = __ldg(rowptr + r);
+                ne = __ldg(rowptr + r + 1);
+            }
+        };
+        const bool skip = one && empty;
+        if (!skip) rows_of(c0 + (int64_t)warp * 32 + lane);
         for (int64_t g0 = c0 + (int64_t)warp * 32; g0 < c1; g0 += BLK_THREADS) {
-            const int64_t r = g0 + lane;
             uint32_t nb = 0;
-            if (!(one && empty)) {
-                int32_t v = -1, s = INT32_MAX, e = 0;
-                if (r < R) {
-                    v = __ldg(id_map + r);
-                    s = __ldg(rowptr + r);
-                    e = __ldg(rowptr + r + 1);
-                }
+            if (!skip) {
+                const int32_t v = nv, s = ns;
+                int32_t e = ne;
+                rows_of(g0 + BLK_THREADS + lane);
                 const bool cand = v >= 0 && !((__ldg(visited + (v >> 5)) >> (v & 31)) & 1u);
                 const unsigned cm = __ballot_sync(0xffffffffu, cand);
-                bool found = false;
                 if (cm != 0u && one && stream) {
                     const int32_t t0 = __shfl_sync(0xffffffffu, s, 0);
                     const int32_t t1 = (int32_t)__reduce_max_sync(0xffffffffu, (unsigned)e);
@@ -240,14 +285,8 @@ __global__ void __launch_bounds__(BLK_THREADS, 2) k_bfs_block_smem(
                     nb = rows & cm;
                 } else if (cm != 0u) {
                     if (!cand) e = s;
-                    const bool serial = cand && e - s < 32;
-                    if (one) {
-                        if (serial)
-                            for (int32_t i = s; i < e && !found; ++i) found = in_slice(sl, __ldg(colidx + i), lo);
-                    } else if (serial) {
-                        found = scan_serial(colidx, s, e, front);
-                    }
-                    found = scan_warp_rows(__ballot_sync(0xffffffffu, cand && !serial), s, e, colidx, front, found);
+                    const bool found = one ? scan_rows(cand, s, e, colidx, SliceBits{sl, lo})
+                                           : scan_rows(cand, s, e, colidx, FrontBits{front});
                     nb = __ballot_sync(0xffffffffu, found);
                 }
             }
@@ -266,7 +305,7 @@ __global__ void __launch_bounds__(BFS_THREADS) k_bfs_merge(const uint32_t *__res
                                                            uint32_t *__restrict__ next, uint32_t *visited,
                                                            int32_t *level, int32_t new_level,
                                                            unsigned long long *count,
-                                                           const int32_t *__restrict__ out_rowptr) {
+                                                           const int32_t *__restrict__ out_rowptr, int split) {
     extern __shared__ uint32_t hit[];  // k/32 words
     __shared__ unsigned long long red[32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -275,32 +314,51 @@ __global__ void __launch_bounds__(BFS_THREADS) k_bfs_merge(const uint32_t *__res
     const int kw = k >> 5;
     for (int t = threadIdx.x; t < kw; t += BFS_THREADS) hit[t] = 0u;
     __syncthreads();
-    for (int32_t b = warp; b < B; b += BFS_WARPS) {
+    // a warp per slice, or (`split`: few blocks, long slices) all warps along each; four rows of a lane in
+    // flight.  8 blocks of a 5M-vertex R-MAT, a level that reaches most vertices: 87 us a warp per slice and a
+    // row at a time, 50 us so
+    const int32_t first = split ? warp * 128 : 0, step = split ? BFS_WARPS * 128 : 128;
+    for (int32_t b = split ? 0 : warp; b < B; b += split ? 1 : BFS_WARPS) {
         const int32_t *o = merge_off + (int64_t)b * (nranges + 1) + j;
         const int32_t r0 = __ldg(o), r1 = __ldg(o + 1);
-        for (int32_t r = r0 + lane; r < r1; r += 32) {
-            if ((__ldg(rowbits + (r >> 5)) >> (r & 31)) & 1u) {
-                const int32_t t = __ldg(id_map + r) - vbase;
-                atomicOr(&hit[t >> 5], 1u << (t & 31));
+        for (int64_t r = (int64_t)r0 + first + lane; r < r1; r += step) {
+            bool set[4];
+            int32_t id[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int64_t q = r + 32 * k;
+                set[k] = q < r1 && ((__ldg(rowbits + (q >> 5)) >> (q & 31)) & 1u);
             }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) id[k] = set[k] ? __ldg(id_map + r + 32 * k) - vbase : 0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (set[k]) atomicOr(&hit[id[k] >> 5], 1u << (id[k] & 31));
         }
     }
     __syncthreads();
+    // a word per lane, then the warp takes its 32 words one by one with a vertex per lane: the level
+    // stores and row offsets are coalesced and independent (a lane walking its own word's bits waited for
+    // every vertex)
     unsigned long long found_total = 0, deg_total = 0;
-    for (int t = threadIdx.x; t < kw; t += BFS_THREADS) {
+    for (int t0 = warp * 32; t0 < kw; t0 += BFS_THREADS) {
+        const int t = t0 + lane;
         const int64_t w = (int64_t)(vbase >> 5) + t;
-        if (w >= nwords) break;
-        const uint32_t vis = visited[w];
-        const uint32_t nb = hit[t] & ~vis;
-        next[w] = nb;
-        if (nb) {
-            visited[w] = vis | nb;
-            found_total += __popc(nb);
-            uint32_t m = nb;
-            while (m) {
-                const int bit = __ffs(m) - 1;
-                m &= m - 1;
-                const int64_t v = w * 32 + bit;
+        uint32_t nb = 0;
+        if (t < kw && w < nwords) {
+            const uint32_t vis = visited[w];
+            nb = hit[t] & ~vis;
+            next[w] = nb;
+            if (nb) visited[w] = vis | nb;
+        }
+        found_total += __popc(nb);
+        unsigned m = __ballot_sync(0xffffffffu, nb != 0u);
+        while (m) {
+            const int l = __ffs(m) - 1;
+            m &= m - 1;
+            const uint32_t x = __shfl_sync(0xffffffffu, nb, l);
+            if ((x >> lane) & 1u) {
+                const int64_t v = ((int64_t)(vbase >> 5) + t0 + l) * 32 + lane;
                 level[v] = new_level;
                 deg_total += (unsigned long long)(__ldg(out_rowptr + v + 1) - __ldg(out_rowptr + v));
             }
@@ -736,23 +794,25 @@ static int res_cluster_size(cudaStream_t s) {
     return chosen;
 }
 
-// Queue of the vertices set in a bitmap (for a push level after a pull level): per word a
-// popcount, an exclusive scan (positions), then the write.
-__global__ void k_bitmap_count(const uint32_t *bits, int32_t nwords, int32_t *cnt) {
-    for (int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; w < nwords; w += (int64_t)gridDim.x * blockDim.x)
-        cnt[w] = __popc(bits[w]);
-}
-
-__global__ void k_bitmap_queue(const uint32_t *bits, int32_t nwords, const int64_t *pos, int32_t *queue) {
-    for (int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; w < nwords; w += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t m = bits[w];
-        int64_t p = pos[w];
+// Queue of the vertices set in a bitmap (for a push level after a pull level), in any order, through the
+// warps' queues: one launch instead of a popcount, a scan and a write (five launches, 17 us).
+__global__ void __launch_bounds__(BFS_THREADS) k_bitmap_queue(const uint32_t *__restrict__ bits, int32_t nwords,
+                                                              int32_t *queue, unsigned long long *count) {
+    __shared__ int32_t wq_buf[BFS_WARPS * WQ_ENTRIES];
+    WarpQueue wq(wq_buf);
+    const int lane = threadIdx.x & 31;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t w0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); w0 < nwords; w0 += step) {
+        const uint32_t mine = w0 + lane < nwords ? __ldg(bits + w0 + lane) : 0u;
+        unsigned m = __ballot_sync(0xffffffffu, mine != 0u);
         while (m) {
-            const int b = __ffs(m) - 1;
+            const int l = __ffs(m) - 1;
             m &= m - 1;
-            queue[p++] = (int32_t)(w * 32 + b);
+            const uint32_t w = __shfl_sync(0xffffffffu, mine, l);
+            wq.push((w >> lane) & 1u, (int32_t)((w0 + l) * 32 + lane), 0, queue, count);
         }
     }
+    wq.finish(queue, count, count);  // no weights: nothing is added to the second word
 }
 
 // edges_reached = sum of out-degrees of vertices with level >= 0; reached = their count.
@@ -856,6 +916,7 @@ static int bfs_impl(const tc_graph *cg, const tc_part *part, int32_t source, con
         TC_CUDA(cudaEventCreate(&lev[0]));
         TC_CUDA(cudaEventCreate(&lev[1]));
     }
+    const int merge_split = part && part->R > (int64_t)part->B * part->nranges * 512 ? 1 : 0;
     const size_t merge_smem = part ? (size_t)(part->k / 32) * 4 : 0;
     // blocked levels with the slice in shared memory: two CTAs per SM
     int blk_grid = 0;
@@ -939,11 +1000,8 @@ static int bfs_impl(const tc_graph *cg, const tc_part *part, int32_t source, con
         push_levels += use_push ? 1 : 0;
         if (use_push) {
             if (!have_queue) {  // frontier came from a pull level: bitmap -> queue
-                k_bitmap_count<<<grid, BFS_THREADS, 0, s>>>(front, nwords, qcnt.as<int32_t>());
+                k_bitmap_queue<<<grid, BFS_THREADS, 0, s>>>(front, nwords, q[lvl & 1], cnt + 2);
                 if (cudaGetLastError() != cudaSuccess) { st = fail(TC_ERR_CUDA, "launch failed"); break; }
-                st = scan_i32_to_i64_ws(qcnt.as<int32_t>(), nwords, qpos.as<int64_t>(), g->ws_scan.as<int64_t>(), s);
-                if (st != TC_OK) break;
-                k_bitmap_queue<<<grid, BFS_THREADS, 0, s>>>(front, nwords, qpos.as<int64_t>(), q[lvl & 1]);
             }
             if (cudaMemsetAsync(next, 0, (size_t)nwords * 4, s) != cudaSuccess) { st = fail(TC_ERR_CUDA, "memset failed"); break; }
             // out-degree prefix of the queue: frontier edges m_f are already known on the host
@@ -976,7 +1034,7 @@ static int bfs_impl(const tc_graph *cg, const tc_part *part, int32_t source, con
                                                                        part->merge_off.as<int32_t>(), part->B,
                                                                        part->nranges, part->k, V, nwords, next,
                                                                        visited, level, lvl + 1, cnt,
-                                                                       g->out_rowptr.as<int32_t>());
+                                                                       g->out_rowptr.as<int32_t>(), merge_split);
             ++tocab_levels;
             have_queue = false;
         } else {

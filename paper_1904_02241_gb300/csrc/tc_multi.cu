@@ -544,7 +544,7 @@ __global__ void k_res_eoff(const int32_t *vtx_off, int32_t n, const int32_t *row
 // first edge gets a head bit.  A warp takes 32 rows at a time: their offsets by coalesced loads, then their
 // edges as one stream, RS_WINDOWS * 32 per step with all loads in flight; an edge's row is the count of rows
 // started up to it (bits of one word per 32 edges).  1,000 R-MAT graphs of scale 10 to 16: a warp per row
-// took 4,713 us, so some 1,200 us.
+// took 4,713 us, so 1,222 us.
 constexpr int RS_THREADS = 256;
 constexpr int RS_WINDOWS = 4;
 __global__ void __launch_bounds__(RS_THREADS) k_res_stream(const int32_t *__restrict__ rowptr,

@@ -899,3 +899,39 @@ def test_partition_of_rows_with_long_gaps(T, order):
     P = T.tocab_partition(G, T.TC_PULL, 3 if order == "natural" else 0, block_policy="smem", order=order)
     assert l1_rel(T.pagerank_pull(G, P).cpu().numpy(), _oracle_pr(g)) <= TOL
     assert l1_rel(T.pagerank_push(G, T.tocab_partition(G, T.TC_PUSH, 2)).cpu().numpy(), _oracle_pr(g)) <= TOL
+
+
+@pytest.mark.parametrize("B", [None, 1, 3])
+def test_pull_level_finds_a_source_at_every_place_of_a_row(T, B):
+    """Pull rows are scanned after 1, 4, 8, ... edges, long ones by their first 16 edges and then by the
+    warp: rows of d in-edges whose only reached source stands at place p."""
+    rows = [(d, p) for d in (1, 2, 3, 4, 5, 8, 9, 16, 17, 31, 32, 33, 47, 48, 49, 79, 80, 81, 96, 100)
+            for p in {0, 1, 3, 4, 5, 15, 16, 17, 31, 32, d // 2, d - 1} if p < d]
+    rows += [(d, None) for d in (1, 4, 31, 32, 80)]  # not reached
+    edges = []
+    for i, (d, p) in enumerate(rows):  # unreached sources 0..99 and 101..200 around the source 100
+        low = d if p is None else p
+        edges += [(u, 201 + i) for u in range(low)]
+        if p is not None:
+            edges += [(100, 201 + i)] + [(101 + u, 201 + i) for u in range(d - 1 - p)]
+    V = 201 + len(rows)
+    g = gg.from_edge_list(V, edges)
+    G = _load(T, g)
+    P = T.tocab_partition(G, T.TC_PULL, B, smem_stage=-1) if B else None
+    rp, ci = g.numpy()
+    lv = T.bfs_pull(G, P, 100, tocab_threshold=0.0 if B else -1.0).cpu().numpy()
+    assert np.array_equal(lv, oracle.bfs(V, rp, ci, 100))
+    assert [int(x) for x in lv[201:]] == [1 if p is not None else -1 for _, p in rows]
+
+
+@pytest.mark.parametrize("B", [1, 2, 40])
+@pytest.mark.parametrize("k", [32, 1024, 8192])
+def test_blocked_bfs_merge_by_slices_of_every_length(T, B, k):
+    """The blocked level's merge gives a slice to a warp, or to the whole CTA where slices are long."""
+    g = gg.symmetrize(gg.rmat(13))
+    G = _load(T, g)
+    P = T.tocab_partition(G, T.TC_PULL, B, merge_range=k, smem_stage=-1)
+    rp, ci = g.numpy()
+    for s in gg.sources(g, 2, seed=3):
+        lv = T.bfs_pull(G, P, s, tocab_threshold=0.0).cpu().numpy()
+        assert np.array_equal(lv, oracle.bfs(g.V, rp, ci, s))
