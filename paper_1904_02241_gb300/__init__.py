@@ -447,5 +447,5 @@ def bfs_pull(graph: Graph, part: Partition | None, source: int, tocab_threshold:
                          int(resident_edges))
     st = L.tc_bfs_stats()
     _check(L.load().tc_bfs_pull(graph.handle, part.handle if part is not None else None, int(source), C.byref(bp),
-                                out.data_ptr(), C.byref(st), _stream(stream)), "tc_bfs_pull")
+                                out.data_ptr(), C.byref(st) if return_stats else None, _stream(stream)), "tc_bfs_pull")
     return (out, st) if return_stats else out

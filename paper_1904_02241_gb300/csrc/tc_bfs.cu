@@ -903,7 +903,7 @@ static int bfs_impl(const tc_graph *cg, const tc_part *part, int32_t source, con
     // direction switching (Beamer et al.): edges out of the frontier (m_f) against edges out of
     // unvisited vertices (m_u); push -> pull when m_f > m_u / 14, pull -> push when the
     // frontier holds fewer than push_threshold * V vertices
-    int32_t sdeg[2] = {0, 0};
+    int32_t *sdeg = reinterpret_cast<int32_t *>(h_cnt);
     TC_CUDA(cudaMemcpyAsync(sdeg, g->out_rowptr.as<int32_t>() + source, 8, cudaMemcpyDeviceToHost, s));
     TC_CUDA(cudaStreamSynchronize(s));
     double m_f = (double)(sdeg[1] - sdeg[0]);
