@@ -227,6 +227,11 @@ struct tc_part {
     bool pperm_built = false, has_vals = false;  // push: values of the matrix (GC-pull SpMV)
     tc::DevBuf pperm;           // int32[E]: the loaded CSR position of every partition entry
     tc::DevBuf pvals;           // float[E]: the matrix values in partition order
+    // staged SpMV (tc_spmv.cu): a finer push partition of the same matrix whose blocks of x fit shared
+    // memory, the loaded CSR position of every staged entry (-1: padding), and the values in that order
+    bool sp_tried = false;
+    tc_part *sp = nullptr;
+    tc::DevBuf sp_perm, sp_vals, sp_err;
     int32_t nptiles = 0;        // push, W * 8 bytes within shared memory: tiles of the staged push
     // push: the edges by destination range of cut_W vertices (fixed-point staged push; tc_push.cu),
     // built on first use
@@ -263,6 +268,7 @@ struct tc_part {
     tc::DevBuf dir_u;           // int32[ndirect + 8]: source (new ID), sorted by target
     tc::DevBuf dir_id16;        // uint16[ndirect + 8]: target minus its range's first vertex
     ~tc_part() {
+        delete sp;
         delete[] h_blk_rows;
         delete[] h_blk_edges;
     }
@@ -285,6 +291,11 @@ int launch_push_smem(const tc_part *p, const float *contrib, void *sums, const f
 int build_tiles(tc_part *p, int sms, cudaStream_t s);
 size_t merge_smem_bytes(int32_t k, int32_t B);   // dynamic shared memory of the ordered pull merge
 size_t merge_atomic_smem_bytes(int32_t k, int32_t B, bool fixed);  // ... of the one-accumulator merges
+// tc_tocab_partition's work on a fresh handle.
+int build_partition(const tc_graph *g, int dir, int32_t num_blocks, const tc_part_params *pp, cudaStream_t s,
+                    tc_part *p);
+// The staged gather with a value per edge: p->partial gets the sums of vals * x.  x needs no alignment.
+int launch_tiled_spmv(const tc_part *p, const float *vals, const float *x, int *err_flag, cudaStream_t s);
 // Launch the staged gather (+ long rows) writing p->partial from contributions `contrib`.
 int launch_tiled_gather(const tc_part *p, const float *contrib, int *err_flag, cudaStream_t s, int *launches);
 

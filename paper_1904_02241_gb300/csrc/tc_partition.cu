@@ -500,8 +500,8 @@ static int weighted_ranges(tc_part *p, int32_t kmax, cudaStream_t s, int grid) {
     return TC_OK;
 }
 
-static int partition_impl(const tc_graph *g, int dir, int32_t num_blocks, const tc_part_params *pp, cudaStream_t s,
-                          tc_part *p) {
+int build_partition(const tc_graph *g, int dir, int32_t num_blocks, const tc_part_params *pp, cudaStream_t s,
+                    tc_part *p) {
     DeviceCaps caps;
     TC_TRY(device_caps(&caps));
     const int32_t V = g->V;
@@ -713,7 +713,7 @@ extern "C" int tc_tocab_partition(const tc_graph *g, int dir, int32_t num_blocks
         return fail(TC_ERR_INVALID_ARG, "tc_tocab_partition: num_blocks must be in [0, V]");
     tc_part *p = new (std::nothrow) tc_part();
     if (!p) return fail(TC_ERR_OOM, "host allocation failed");
-    int st = partition_impl(g, dir, num_blocks, params, (cudaStream_t)stream, p);
+    int st = build_partition(g, dir, num_blocks, params, (cudaStream_t)stream, p);
     if (st != TC_OK) {
         cudaStreamSynchronize((cudaStream_t)stream);
         delete p;

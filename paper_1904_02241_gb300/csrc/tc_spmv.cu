@@ -6,6 +6,8 @@
 // than the graph's hub degree, 2048 by default).  Each lane strides its row's entries
 // (coalesced column and value loads, random gathers of x) and a fixed shuffle / shared-memory
 // tree adds the lane sums, so the result does not depend on timing.  FP32 throughout.
+#include <vector>
+
 #include "tc_internal.cuh"
 
 namespace tc {
@@ -171,6 +173,184 @@ __global__ void __launch_bounds__(SP_THREADS) k_spmv_merge(const float *__restri
     }
 }
 
+// Staged GC-pull.  With blocks of x that only fit the L2, an entry costs a random L2 request, and those
+// come at some 190 G/s whatever the order of the rows.  So from SPM_MIN_ENTRIES entries on (below, the
+// launches dominate either way), where it pays, the values get a finer cut of the matrix whose blocks of x
+// fit one CTA's shared memory, in the staged form of the rank gather (tc_tile.cu) with a value per entry:
+// the entries stream at 6 B each and x is read in shared memory.
+// More pieces come with it, so their merge is a kernel of its own.  R-MAT 22, 8 blocks: 404 us the general
+// way; 129 us for the staged gather and 95 us for the merge, whose 64-bit shared reads and writes at random
+// rows bound it (bank conflicts).  R-MAT of 131,072 rows, 16 blocks: 57 to 32 us.
+//
+// CTA j owns rows [j k, (j+1) k).  The order is the same fixed one as k_spmv_merge's, block after block
+// with a barrier, but a thread's entries (SPAN per block) of the next DEPTH blocks load while those of
+// the DEPTH blocks before are added.
+// There are several times the pieces of the loaded blocks, so the additions are compensated (the error of
+// every one, by Knuth's TwoSum, is added up beside the sum): without it y was further from the exact
+// product than with eight blocks (R-MAT 22: 1.7e-7 against 9.9e-8 in the 2-norm).
+constexpr int SPM_THREADS = 512;
+constexpr int64_t SPM_MIN_ENTRIES = 1 << 20;
+__device__ __forceinline__ void spm_add(float2 *acc, float v) {  // x: the sum, y: its error
+    const float2 a = *acc;
+    const float t = a.x + v;
+    const float z = t - a.x;
+    *acc = make_float2(t, a.y + ((a.x - (t - z)) + (v - z)));
+}
+template <int DEPTH, int SPAN>
+__global__ void __launch_bounds__(SPM_THREADS, DEPTH * SPAN <= 4 ? 4 : 2) k_spmv_merge_staged(const float *__restrict__ partial,
+                                                                   const uint16_t *__restrict__ id16,
+                                                                   const int32_t *__restrict__ offT, int32_t B,
+                                                                   int32_t k, int32_t V, const int *err, float *y) {
+    extern __shared__ float2 sacc[];  // [k], then block b's rows of the range, [off[b], off[B + b])
+    int32_t *off = reinterpret_cast<int32_t *>(sacc + k);
+    const int32_t j = blockIdx.x;
+    for (int32_t t = threadIdx.x; t < k; t += SPM_THREADS) sacc[t] = make_float2(0.0f, 0.0f);
+    for (int32_t b = threadIdx.x; b < 2 * B; b += SPM_THREADS) off[b] = __ldg(offT + (int64_t)j * B + b);
+    __syncthreads();
+    float va[DEPTH][SPAN], vb[DEPTH][SPAN];
+    uint32_t ia[DEPTH][SPAN], ib[DEPTH][SPAN];
+    auto load = [&](int32_t b0, float(&v)[DEPTH][SPAN], uint32_t(&id)[DEPTH][SPAN]) {
+#pragma unroll
+        for (int q = 0; q < DEPTH; ++q)
+#pragma unroll
+            for (int h = 0; h < SPAN; ++h) {
+                id[q][h] = ~0u;
+                if (b0 + q < B) {
+                    const int32_t r = off[b0 + q] + (int32_t)threadIdx.x + h * SPM_THREADS;
+                    if (r < off[B + b0 + q]) {
+                        v[q][h] = __ldcs(partial + r);
+                        id[q][h] = __ldcs(id16 + r);
+                    }
+                }
+            }
+    };
+    auto add = [&](int32_t b0, float(&v)[DEPTH][SPAN], uint32_t(&id)[DEPTH][SPAN]) {
+#pragma unroll
+        for (int q = 0; q < DEPTH; ++q) {
+            if (b0 + q >= B) break;
+#pragma unroll
+            for (int h = 0; h < SPAN; ++h)
+                if (id[q][h] != ~0u) spm_add(sacc + id[q][h], v[q][h]);
+            for (int32_t r = off[b0 + q] + (int32_t)threadIdx.x + SPAN * SPM_THREADS; r < off[B + b0 + q]; r += SPM_THREADS)
+                spm_add(sacc + __ldcs(id16 + r), __ldcs(partial + r));
+            __syncthreads();  // before the next block's
+        }
+    };
+    load(0, va, ia);
+    for (int32_t b0 = 0; b0 < B; b0 += 2 * DEPTH) {
+        load(b0 + DEPTH, vb, ib);
+        add(b0, va, ia);
+        load(b0 + 2 * DEPTH, va, ia);
+        add(b0 + DEPTH, vb, ib);
+    }
+    const bool bad = *err != 0;  // a bounded wait of the gather gave up: no sum is right
+    for (int32_t t = threadIdx.x; t < k && (int64_t)j * k + t < V; t += SPM_THREADS) {
+        const float2 a = sacc[t];
+        const float sum = fabsf(a.x) <= 3.402823466e38f ? a.x + a.y : a.x;  // infinities and NaN as they are
+        y[(int64_t)j * k + t] = bad ? __int_as_float(0x7fffffff) : sum;
+    }
+}
+
+static size_t spm_smem_bytes(const tc_part *sp) { return (size_t)sp->k * 8 + (size_t)sp->B * 8; }
+
+// perm into the staged order: entry i of block b goes to i + delta[b].
+__global__ void k_stage_perm(const int32_t *__restrict__ colidx, const int32_t *__restrict__ perm, int64_t E, DivBy W,
+                             const int64_t *__restrict__ delta, int32_t *__restrict__ out) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < E; i += (int64_t)gridDim.x * blockDim.x)
+        out[i + __ldg(delta + div_apply(colidx[i], W))] = perm[i];
+}
+
+__global__ void k_gather_vals_staged(const int32_t *__restrict__ perm, const float *__restrict__ vals, int64_t n,
+                                     float *__restrict__ out) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        out[i] = perm[i] >= 0 ? vals[perm[i]] : 0.0f;
+}
+
+// How often consecutive entries change the block: about the pieces of a cut into blocks of W columns.
+__global__ void __launch_bounds__(SP_THREADS) k_block_changes(const int32_t *__restrict__ colidx, int64_t E, DivBy W,
+                                                              unsigned long long *count) {
+    unsigned n = 0;
+    for (int64_t i = blockIdx.x * (int64_t)SP_THREADS + threadIdx.x; i < E; i += (int64_t)gridDim.x * SP_THREADS)
+        n += i == 0 || div_apply(__ldg(colidx + i), W) != div_apply(__ldg(colidx + i - 1), W) ? 1u : 0u;
+    n = __reduce_add_sync(0xffffffffu, n);
+    if ((threadIdx.x & 31) == 0 && n) atomicAdd(count, (unsigned long long)n);
+}
+
+// Does the staged form pay?  Its gather is always the faster one, its merge has more pieces: where nearly
+// every entry becomes a piece and the loaded blocks have few of them, the merge takes what the gather gains.
+// Pieces beyond the loaded ones, of the entries, and times against the general form: uniform matrix of 16
+// entries per row, 4 blocks: 0.51 (1M rows) 101 against 136 us, 0.61 (2M) 188 / 206, 0.68 (4M) 370 / 354, 0.71
+// (8M) 736 / 694; with 16 blocks 0.33 (8M) 735 / 840; R-MAT 22 with 8 blocks below 0.4, 245 / 404.
+static int staged_pays(const tc_part *p, int32_t W, const DeviceCaps &caps, cudaStream_t s, bool *pays) {
+    DevBuf cnt;
+    TC_TRY(cnt.alloc(8));
+    TC_CUDA(cudaMemsetAsync(cnt.p, 0, 8, s));
+    k_block_changes<<<caps.sms * 8, SP_THREADS, 0, s>>>(p->g->out_colidx.as<int32_t>(), p->E, div_by(W),
+                                                        cnt.as<unsigned long long>());
+    TC_LAUNCH_CHECK();
+    unsigned long long n = 0;
+    TC_CUDA(cudaMemcpyAsync(&n, cnt.p, 8, cudaMemcpyDeviceToHost, s));
+    TC_CUDA(cudaStreamSynchronize(s));
+    *pays = (double)n - (double)p->R < 0.63 * (double)p->E;
+    return TC_OK;
+}
+
+// The staged form of push partition p's matrix into `sp` and p->sp_perm, sp_vals, sp_err.
+static int build_staged(tc_part *p, tc_part *sp, const DeviceCaps &caps, cudaStream_t s) {
+    const int64_t E = p->E;
+    const int32_t *ci = p->g->out_colidx.as<int32_t>();
+    const int32_t wmax = tile_max_width(caps.max_smem_optin);
+    tc_part_params pp = {};
+    pp.smem_stage = -1;
+    const int32_t nb = (int32_t)(((int64_t)p->V + wmax - 1) / wmax);
+    bool pays = false;
+    TC_TRY(staged_pays(p, (p->V + nb - 1) / nb, caps, s, &pays));
+    if (!pays) return fail(TC_ERR_UNSUPPORTED, "build_staged: too many pieces");
+    TC_TRY(build_partition(p->g, TC_PUSH, nb, &pp, s, sp));
+    if (sp->W > wmax || sp->W % 32 != 0 || !sp->id16.p || spm_smem_bytes(sp) > (size_t)caps.max_smem_optin) return fail(TC_ERR_UNSUPPORTED, "build_staged: width");
+    TC_TRY(build_tiles(sp, caps.sms, s));
+    if (!sp->tiled) return fail(TC_ERR_UNSUPPORTED, "build_staged: no staged form");
+    DevBuf iota, keys, perm, kt, vt, delta;
+    TC_TRY(iota.alloc((size_t)E * 4));
+    k_iota<<<caps.sms * 8, 256, 0, s>>>(E, iota.as<int32_t>());
+    TC_LAUNCH_CHECK();
+    if (sp->B > 1) {  // the partition's own stable sort, carrying each entry's position
+        TC_TRY(keys.alloc((size_t)E * 4));
+        TC_TRY(perm.alloc((size_t)E * 4));
+        TC_TRY(kt.alloc((size_t)E * 4));
+        TC_TRY(vt.alloc((size_t)E * 4));
+        int bits = 0;
+        while ((1LL << bits) < (int64_t)sp->B) ++bits;
+        TC_TRY(stable_bucket_sort(ci, iota.as<int32_t>(), keys.as<int32_t>(), perm.as<int32_t>(), kt.as<int32_t>(),
+                                  vt.as<int32_t>(), E, sp->W, bits, s));
+    } else {
+        perm.swap(iota);
+    }
+    std::vector<int64_t> h_delta((size_t)sp->B);
+    int64_t pb = 0;
+    for (int32_t b = 0; b < sp->B; ++b) {
+        h_delta[(size_t)b] = pb - sp->h_blk_edges[b];
+        pb += (sp->h_blk_edges[b + 1] - sp->h_blk_edges[b] + TILE_WCHUNK - 1) / TILE_WCHUNK * TILE_WCHUNK;
+    }
+    const int64_t n = sp->padded_edges + TILE_WCHUNK;  // with the chunk of slack of the staged stream
+    TC_TRY(delta.alloc(h_delta.size() * 8));
+    TC_TRY(p->sp_perm.alloc((size_t)n * 4));
+    TC_TRY(p->sp_vals.alloc((size_t)n * 4));
+    TC_TRY(p->sp_err.alloc(4));
+    TC_CUDA(cudaMemsetAsync(p->sp_err.p, 0, 4, s));
+    TC_CUDA(cudaMemsetAsync(p->sp_perm.p, 0xFF, (size_t)n * 4, s));
+    TC_CUDA(cudaMemcpyAsync(delta.p, h_delta.data(), h_delta.size() * 8, cudaMemcpyHostToDevice, s));
+    k_stage_perm<<<caps.sms * 8, 256, 0, s>>>(sp->colidx.as<int32_t>(), perm.as<int32_t>(), E, div_by(sp->W),
+                                              delta.as<int64_t>(), p->sp_perm.as<int32_t>());
+    TC_LAUNCH_CHECK();
+    TC_CUDA(cudaStreamSynchronize(s));
+    // the gather and the merge need neither of these
+    for (DevBuf *d : {&sp->colidx, &sp->esrc, &sp->rowptr, &sp->id_map, &sp->rowbits, &sp->merge_off, &sp->merge_gpre,
+                      &sp->hubs})
+        d->release();
+    return TC_OK;
+}
+
 // GC-push (Sec. 4's SpMV in the push direction with TOCAB): the pieces of a TC_PULL partition of
 // the matrix's graph.  Piece r = (row block b, column j = id_map[r]) holds the entries (i, j) of
 // A with i in block b; x[j] is read once per piece and every entry adds vals * x[j] into y[i]
@@ -221,6 +401,31 @@ extern "C" int tc_part_set_values(tc_part *p, const float *vals, int mem, void *
     DeviceCaps caps;
     TC_TRY(device_caps(&caps));
     const int grid = caps.sms * 8;
+    // Not under a memory cap, and not where its memory is not to be had: the general form needs less.
+    if (!p->sp_tried && p->dir == TC_PUSH && E >= SPM_MIN_ENTRIES && !cache_get_limit()) {
+        p->sp_tried = true;
+        tc_part *sp = new (std::nothrow) tc_part();
+        if (sp) {
+            const int st = build_staged(p, sp, caps, s);
+            if (st == TC_OK) {
+                p->sp = sp;
+            } else {
+                TC_CUDA(cudaStreamSynchronize(s));
+                delete sp;
+                p->sp_perm.release();
+                p->sp_vals.release();
+                if (st != TC_ERR_OOM && st != TC_ERR_UNSUPPORTED) return st;
+            }
+        }
+    }
+    if (p->sp) {
+        k_gather_vals_staged<<<grid, 256, 0, s>>>(p->sp_perm.as<int32_t>(), vals, p->sp->padded_edges + TILE_WCHUNK,
+                                                  p->sp_vals.as<float>());
+        TC_LAUNCH_CHECK();
+        TC_CUDA(cudaStreamSynchronize(s));
+        p->has_vals = true;
+        return TC_OK;
+    }
     if (!p->pperm_built) {  // the partition's own sorts again, carrying each entry's position
         TC_TRY(p->pperm.alloc((size_t)(E > 0 ? E : 1) * 4));
         if (E > 0) {
@@ -289,6 +494,23 @@ extern "C" int tc_spmv_tocab(const tc_part *p, const float *x, float *y, int mem
         return TC_OK;
     }
     if ((size_t)p->k * 4 > 200 * 1024) return fail(TC_ERR_UNSUPPORTED, "tc_spmv_tocab: merge_range above 51,200");
+    if (p->sp) {
+        const tc_part *sp = p->sp;
+        TC_TRY(launch_tiled_spmv(sp, p->sp_vals.as<float>(), x, p->sp_err.as<int>(), (cudaStream_t)stream));
+        // entries per thread and block: one, two or four, by the mean slice of a block and range (an entry
+        // past them is a round trip of its own)
+        const int64_t slice = sp->R / ((int64_t)sp->B * sp->nranges);
+        auto merge = slice <= SPM_THREADS * 3 / 4   ? k_spmv_merge_staged<4, 1>
+                     : slice <= SPM_THREADS * 7 / 4 ? k_spmv_merge_staged<4, 2>
+                                                    : k_spmv_merge_staged<2, 4>;
+        const size_t smem = spm_smem_bytes(sp);
+        TC_CUDA(cudaFuncSetAttribute(merge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        merge<<<sp->nranges, SPM_THREADS, smem, (cudaStream_t)stream>>>(
+            sp->partial.as<float>(), sp->id16.as<uint16_t>(), sp->merge_offT.as<int32_t>(), sp->B, sp->k, V,
+            p->sp_err.as<int>(), y);
+        TC_LAUNCH_CHECK();
+        return TC_OK;
+    }
     DeviceCaps caps;
     TC_TRY(device_caps(&caps));
     cudaStream_t s = (cudaStream_t)stream;

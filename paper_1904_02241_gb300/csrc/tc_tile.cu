@@ -61,6 +61,7 @@ struct TileArgs {
     int32_t V, W;
     float *partial;
     int *err;
+    const float *vals;       // a value per staged edge (SpMV; null in the rank gather)
 };
 
 // Loads lane `lane`'s 16 staged edges of the chunk at q0 (sources and row-start bits).
@@ -75,6 +76,8 @@ __device__ __forceinline__ void load_chunk(const TileArgs &t, int32_t q0, int la
 // One warp's row-aligned range: edges [es, ee) of the staged stream, whose first row rs starts
 // at es (Alg. 4 on the block values in `slice`); every row of it goes to partial[].
 // Software pipeline: every chunk's loads are issued before the previous one is summed.
+// VALS: an edge adds its value times the source's (one rounding per edge: fused multiply-adds).
+template <bool VALS>
 __device__ __forceinline__ void warp_walk(const TileArgs &t, const float *slice, float *stage_base, int32_t es,
                                           int32_t ee, int32_t rs, int lane) {
     int32_t rowbase = rs;                 // row started by the next head
@@ -93,12 +96,27 @@ __device__ __forceinline__ void warp_walk(const TileArgs &t, const float *slice,
         const uint4 c0 = nc0, c1 = nc1;
         uint32_t hd = nh;
         if (q0 + WCH < ee) load_chunk(t, q0 + WCH, lane, nc0, nc1, nh);
+        float vv[16];
+        if (VALS) {
+            const float4 *pv = reinterpret_cast<const float4 *>(t.vals + q0 + 16 * lane);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float4 f = __ldcs(pv + i);
+                vv[4 * i] = f.x;
+                vv[4 * i + 1] = f.y;
+                vv[4 * i + 2] = f.z;
+                vv[4 * i + 3] = f.w;
+            }
+        }
         const uint32_t words[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
         const bool full = q0 >= es && q0 + WCH <= ee;  // whole chunk inside the warp's range (warp-uniform)
         if (full && __ballot_sync(0xffffffffu, hd != 0u) == 0u) {
             float s4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-            for (int i = 0; i < 16; ++i) s4[i & 3] += slice[(words[i >> 1] >> (16 * (i & 1))) & 0xFFFFu];
+            for (int i = 0; i < 16; ++i) {
+                const float x = slice[(words[i >> 1] >> (16 * (i & 1))) & 0xFFFFu];
+                s4[i & 3] = VALS ? fmaf(vv[i], x, s4[i & 3]) : s4[i & 3] + x;
+            }
             racc += (s4[0] + s4[1]) + (s4[2] + s4[3]);
             pend = true;
             continue;
@@ -127,6 +145,7 @@ __device__ __forceinline__ void warp_walk(const TileArgs &t, const float *slice,
             for (int i = 0; i < 16; ++i) {
                 const uint32_t col = (words[i >> 1] >> (16 * (i & 1))) & 0xFFFFu;
                 val[i] = ((valid >> i) & 1u) ? slice[col] : 0.0f;
+                if (VALS && !((valid >> i) & 1u)) vv[i] = 0.0f;
             }
         }
         // rows of this chunk: exclusive scan of head counts over lanes, from bit-sliced ballots
@@ -156,7 +175,9 @@ __device__ __forceinline__ void warp_walk(const TileArgs &t, const float *slice,
         for (int i = 0; i < 16; ++i) {
             if ((close_m >> i) & 1u) *out++ = seg;  // close the row before this head
             if ((first_m >> i) & 1u) first = seg;   // the piece before the first head
-            seg = ((hd >> i) & 1u) ? val[i] : seg + val[i];
+            const bool head = (hd >> i) & 1u;
+            if (VALS) seg = fmaf(vv[i], val[i], head ? 0.0f : seg);
+            else seg = head ? val[i] : seg + val[i];
         }
         const bool seen = hd != 0u;
         if (!seen) first = seg;
@@ -244,8 +265,44 @@ __global__ void __launch_bounds__(TILE_THREADS, 1) k_tile_gather(TileArgs t) {
     if (!mbar_wait(&slice_bar, 0, t.err, 1)) return;
     const int2 w0 = t.wtab[(int64_t)tile * (TWARPS + 1) + warp];
     const int2 w1 = t.wtab[(int64_t)tile * (TWARPS + 1) + warp + 1];
-    if (w0.x < w1.x) warp_walk(t, slice, stage_base, w0.x, w1.x, w0.y, lane);
+    if (w0.x < w1.x) warp_walk<false>(t, slice, stage_base, w0.x, w1.x, w0.y, lane);
     if (lane == 0) bulk_store_wait_all();  // the stage must outlive the bulk stores reading it
+}
+
+// The same gather for the SpMV.  The block's x comes from the caller's buffer, which may start anywhere
+// and ends at V: bulk copies for what is 16-byte aligned, plain loads for the rest.
+__global__ void __launch_bounds__(TILE_THREADS, 1) k_tile_spmv(TileArgs t) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ __align__(8) uint64_t slice_bar;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int32_t b = t.tile_blk[blockIdx.x];
+    float *slice = reinterpret_cast<float *>(smem);
+    float *stage_base = reinterpret_cast<float *>(smem + slice_bytes(t.W)) + warp * WSTAGE;
+    if (tid == 0) {
+        mbar_init(&slice_bar, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    const int64_t lo = (int64_t)b * t.W;
+    const int32_t n = (int32_t)(((int64_t)t.V - lo) < t.W ? ((int64_t)t.V - lo) : t.W);
+    const float *src = t.contrib + lo;
+    const int32_t nbulk = (reinterpret_cast<uintptr_t>(src) & 15) ? 0 : n & ~3;
+    if (tid == 0 && nbulk > 0) {
+        const uint32_t bytes = (uint32_t)nbulk * 4u;
+        mbar_expect_tx(&slice_bar, bytes);
+        for (uint32_t off = 0; off < bytes; off += 16384) {
+            const uint32_t part = (bytes - off) < 16384u ? (bytes - off) : 16384u;
+            bulk_g2s(reinterpret_cast<unsigned char *>(slice) + off,
+                     reinterpret_cast<const unsigned char *>(src) + off, part, &slice_bar);
+        }
+    }
+    for (int32_t i = nbulk + tid; i < n; i += TILE_THREADS) slice[i] = __ldg(src + i);
+    __syncthreads();
+    if (nbulk > 0 && !mbar_wait(&slice_bar, 0, t.err, 1)) return;
+    const int2 w0 = t.wtab[(int64_t)blockIdx.x * (TWARPS + 1) + warp];
+    const int2 w1 = t.wtab[(int64_t)blockIdx.x * (TWARPS + 1) + warp + 1];
+    if (w0.x < w1.x) warp_walk<true>(t, slice, stage_base, w0.x, w1.x, w0.y, lane);
+    if (lane == 0) bulk_store_wait_all();
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -537,6 +594,7 @@ int launch_tiled_gather(const tc_part *p, const float *contrib, int *err_flag, c
     t.W = p->W;
     t.partial = const_cast<float *>(p->partial.as<float>());
     t.err = err_flag;
+    t.vals = nullptr;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(p->ntiles);
     cfg.blockDim = dim3(TILE_THREADS);
@@ -549,6 +607,25 @@ int launch_tiled_gather(const tc_part *p, const float *contrib, int *err_flag, c
     cfg.numAttrs = 1;
     TC_CUDA(cudaLaunchKernelEx(&cfg, k_tile_gather, t));
     ++*launches;
+    return TC_OK;
+}
+
+int launch_tiled_spmv(const tc_part *p, const float *vals, const float *x, int *err_flag, cudaStream_t s) {
+    const size_t smem = tile_smem_bytes(p->W);
+    TC_CUDA(cudaFuncSetAttribute(k_tile_spmv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    TileArgs t;
+    t.col16 = p->col16.as<uint16_t>();
+    t.heads = p->heads.as<uint16_t>();
+    t.tile_blk = p->tile_blk.as<int32_t>();
+    t.wtab = p->wtab.as<int2>();
+    t.contrib = x;
+    t.V = p->V;
+    t.W = p->W;
+    t.partial = p->partial.as<float>();
+    t.err = err_flag;
+    t.vals = vals;
+    k_tile_spmv<<<p->ntiles, TILE_THREADS, smem, s>>>(t);
+    TC_LAUNCH_CHECK();
     return TC_OK;
 }
 

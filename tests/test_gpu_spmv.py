@@ -224,3 +224,51 @@ def test_tocab_spmv_on_degenerate_matrices(T, d):
         if g.E:
             want[2] = 1.5 * 1.0  # row 2 holds one entry in column 0
         np.testing.assert_array_equal(y, want)
+
+
+def _big_matrix(V, entries, seed):
+    """Exactly `entries` distinct entries: a row and a column with many, a band of empty rows, the rest random."""
+    rng = np.random.default_rng(seed)
+    n = entries * 2
+    rows = rng.integers(0, V, n)
+    rows[(rows > V // 3) & (rows < V // 2)] = V - 1
+    cols = rng.integers(0, V, n)
+    cols[: n // 16] = V // 5
+    key = np.unique((rows.astype(np.int64) * V + cols)[rows != cols])  # the generator drops the diagonal
+    key = np.sort(rng.permutation(key)[:entries])
+    assert key.size == entries
+    g = gg.from_edge_list(V, np.stack([key // V, key % V], axis=1))
+    assert g.colidx.numel() == entries
+    return g
+
+
+@pytest.mark.parametrize("V,entries,B", [(41344, (1 << 20) + 3, 4), (41345, 1 << 20, 1), (130003, (1 << 20) - 1, 8),
+                                         (130003, 1 << 20, 8), (700001, 1300000, 16)])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_staged_gc_pull_matches_oracle_within_the_fp32_bound(T, V, entries, B, shift):
+    """From 2^20 entries on the values also get the staged form (x in shared memory by blocks of 41,344
+    columns, compensated merge): around that line and that width, with x off the 16-byte boundary.  The
+    longest chain of a row has no more roundings than it has entries and a dozen (the warp's scan, the
+    merge's last addition)."""
+    g = _big_matrix(V, entries, V + entries)
+    rng = np.random.default_rng(5)
+    vals = torch.from_numpy(rng.standard_normal(entries).astype(np.float32))
+    buf = torch.from_numpy(rng.standard_normal(V + 1).astype(np.float32))
+    x = buf[shift:shift + V]
+    G = T.graph_load_csr(g.rowptr.cuda(), g.colidx.cuda(), V=V)
+    P = T.tocab_partition(G, T.TC_PUSH, B)
+    T.part_set_values(P, vals.cuda())
+    xd = buf.cuda()[shift:shift + V]
+    y = T.spmv_tocab(P, xd).cpu().numpy().astype(np.float64)
+    rp, ci = g.numpy()
+    v64, x64 = vals.numpy().astype(np.float64), x.numpy().astype(np.float64)
+    want, mag = oracle.spmv(V, rp, ci, v64, x64), oracle.spmv(V, rp, ci, np.abs(v64), np.abs(x64))
+    bound = (np.diff(rp) + 12) * 2.0 ** -24 * mag
+    assert np.all(np.abs(y - want) <= bound + 1e-30)
+    assert np.array_equal(y, T.spmv_tocab(P, xd).cpu().numpy().astype(np.float64))
+    T.part_set_values(P, 2.0 * vals.cuda())  # new values of the same matrix: scaled exactly
+    assert np.array_equal(2.0 * y, T.spmv_tocab(P, xd).cpu().numpy().astype(np.float64))
+    xd[V // 5] = float("inf")  # the column with many entries: its rows alone stop being finite
+    hit = np.zeros(V, dtype=bool)
+    hit[np.repeat(np.arange(V), np.diff(rp))[ci == V // 5]] = True
+    assert np.array_equal(~np.isfinite(T.spmv_tocab(P, xd).cpu().numpy()), hit)
