@@ -159,33 +159,29 @@ __device__ __forceinline__ void warp_walk(const TileArgs &t, const float *slice,
             before += __popc(m & lt_mask) << bit;
             total += __popc(m) << bit;
         }
-        // walk the lane's 16 edges (branch-free): the piece before the first head goes to the
-        // carry scan; every later head closes a whole row, written to the stage
+        // walk the lane's 16 edges (branch-free): every head closes a row, written to the stage (the
+        // lane's first one without what earlier lanes and chunks hold of its row, added below)
         // stage[i] holds row rowbase - 1 + i; it starts (rowbase - 1) mod 4 floats into the
         // warp's buffer so that stage and partial[] agree modulo 16 bytes.  The previous
         // chunk's bulk store must have finished reading the buffer before it is rewritten.
         float *stage = stage_base + ((rowbase - 1) & 3);
         if (lane == 0) bulk_store_wait_read();
         __syncwarp();
-        float seg = 0.0f, first = 0.0f;
-        float *out = stage + before + 1;
-        const uint32_t close_m = hd & (hd - 1u);  // heads after the lane's first: each closes a row
-        const uint32_t first_m = hd & (0u - hd);  // the lane's first head
+        float seg = 0.0f;
+        float *out = stage + before;
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
-            if ((close_m >> i) & 1u) *out++ = seg;  // close the row before this head
-            if ((first_m >> i) & 1u) first = seg;   // the piece before the first head
             const bool head = (hd >> i) & 1u;
+            if (head) *out++ = seg;  // close the row before this head
             if (VALS) seg = fmaf(vv[i], val[i], head ? 0.0f : seg);
             else seg = head ? val[i] : seg + val[i];
         }
         const bool seen = hd != 0u;
-        if (!seen) first = seg;
         // carry of the open row across lanes: segmented inclusive scan (Hillis-Steele). The
         // flag of lane l after the step of distance d is "a head in lanes (l - 2d, l]", read
         // from one ballot of the heads instead of being shuffled along with the values.
         const uint32_t F = __ballot_sync(0xffffffffu, seen);
-        float v = seg;  // the open row's value at the lane's end (== first when no head)
+        float v = seg;  // the open row's value at the lane's end
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
             const float vp = __shfl_up_sync(0xffffffffu, v, d);
@@ -195,11 +191,12 @@ __device__ __forceinline__ void warp_walk(const TileArgs &t, const float *slice,
         }
         const bool f = (F & ((2u << lane) - 1u)) != 0u;  // a head in lanes [0, lane]
         // open-row value at the end of lane l: f ? v : carry + v (no head yet: the chunk's
-        // carry flows through); the row closed at lane l's first head gets X(l-1) + first
+        // carry flows through); the row closed at lane l's first head gets X(l-1) on top of the piece
+        // before that head, which the walk has left in its place
         const float vprev = __shfl_up_sync(0xffffffffu, v, 1);
         const bool fprev = (F & lt_mask) != 0u;
         const float xprev = (lane == 0) ? carry : (fprev ? vprev : carry + vprev);
-        if (seen) stage[before] = xprev + first;
+        if (seen) stage[before] += xprev;
         const float xlast = __shfl_sync(0xffffffffu, f ? v : carry + v, 31);
         // Rows rowbase - 1 + [i0, total) leave: stage[0] is the open row only when it belongs
         // to this warp.  The 16-byte aligned middle goes out as one bulk store (TMA) issued by
