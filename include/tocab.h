@@ -278,11 +278,12 @@ typedef struct tc_pr_params {
     int32_t lb_warp_min;      /* unstaged gathers (Sec. 3.2): rows with fewer edges are summed
                                  by one lane, longer rows by a warp (hubs by a CTA); 0 = 32,
                                  1 = a warp for every row, large = lane-serial; a partition's
-                                 per-block table (tc_part_set_lb) overrides it.  Push: 0 = an
-                                 edge-parallel scatter (a thread per edge, the default; with a
-                                 partition whose destination range fits shared memory, the
-                                 staged scatter of tc_push.cu), > 0 = that thread/warp/CTA row
-                                 mapping (TWC) with this threshold */
+                                 per-block table (tc_part_set_lb) overrides it.  Push: 0 = the
+                                 default (with a partition and fixed-point sums, by destination
+                                 ranges in shared memory with the update fused, tc_push.cu; else
+                                 a thread per edge), > 0 = that thread/warp/CTA row mapping
+                                 (TWC) with this threshold.  Fixed-point sums give the same bits
+                                 either way */
     int32_t l2_window;        /* nonzero: unstaged pull gathers (unblocked, or a partition without
                                  the staged format) run with an L2 access-policy window over the
                                  contributions they read, so that the cache keeps the block's
@@ -525,7 +526,10 @@ int tc_spmv(const tc_graph *g, const float *vals, const float *x, float *y, int 
  * TC_PULL partition's blocks are ranges of W rows of A and its local rows the (row block,
  * column) pieces (GC-push SpMV).  The partition keeps the values in its own entry order (the
  * first call also records that order: the partition's stable sorts again, carrying entry
- * positions).  For the SpMV of Sec. 4.  Synchronises.
+ * positions).  From 2^20 entries on a TC_PUSH partition may keep them in a finer cut instead, whose
+ * blocks of x fit one CTA's shared memory (built by the first call; not under a memory limit, nor
+ * where its memory is not to be had or its pieces would cost more than it gains).  For the SpMV of
+ * Sec. 4.  Synchronises.
  * Errors: TC_ERR_INVALID_ARG (NULL), TC_ERR_UNSUPPORTED (host values, a renumbered partition),
  * TC_ERR_OOM, TC_ERR_CUDA.
  */
@@ -536,12 +540,14 @@ int tc_part_set_values(tc_part *p, const float *vals, int mem, void *stream);
  *   TC_PUSH partition: GC-pull.  For every local row (column block b, row i), partial = sum of
  *       vals * x[col] over the piece's entries (x's block b is the working set, Sec. 3.1), then
  *       the merge of Fig. 5 adds row i's pieces in block order.  FP32 in a fixed order
- *       (deterministic).  The merge_range k must be at most 51,200.
+ *       (deterministic); with the finer cut of tc_part_set_values in that cut's order, the pieces
+ *       added with compensation.  The merge_range k must be at most 51,200.
  *   TC_PULL partition (graph's own numbering): GC-push.  y = 0, then for every local row (row
  *       block b, column j) each entry (i, j) adds vals * x[j] into y[i] with an FP32 atomic add
  *       (y's block b is the working set).  The order of the additions depends on timing, so the
  *       last bits of y may differ between calls; each y[i] is within the FP32 summation bound.
- *   In both, a lane takes a piece below 32 entries, a warp a longer one (Sec. 3.2).
+ *   In both, a lane takes a piece below 32 entries, a warp a longer one (Sec. 3.2); the finer cut's
+ *   pieces are walked as one stream.
  *   p : a partition of the graph holding A, with values set by tc_part_set_values.
  *   x : float[V], y : float[V], device.
  * Asynchronous on `stream`.  Errors: TC_ERR_INVALID_ARG, TC_ERR_UNSUPPORTED, TC_ERR_CUDA.
