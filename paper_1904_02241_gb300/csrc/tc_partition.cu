@@ -158,14 +158,26 @@ __global__ void k_order_apply(const int32_t *perm, const int32_t *in_rowptr, con
 }
 
 // Renumbered G^T: edge e of new row n is edge (e - rowptr_new[n]) of old row perm[n], with its
-// source renumbered.  Sources keep the old row's order (ascending old ID).
-__global__ void k_order_edges(const int32_t *row_of_edge, const int32_t *rowptr_new, const int32_t *perm,
-                              const int32_t *in_rowptr, const int32_t *in_colidx, const int32_t *inv, int64_t E,
-                              int32_t *colidx_new) {
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < E; e += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t n = row_of_edge[e];
-        const int64_t src_pos = (int64_t)in_rowptr[perm[n]] + (e - rowptr_new[n]);
-        colidx_new[e] = inv[in_colidx[src_pos]];
+// source renumbered.  Sources keep the old row's order (ascending old ID).  A chain of four dependent
+// reads per edge, so a thread keeps four edges in flight (64M edges: 384 us one by one, 316 us so).
+__global__ void k_order_edges(const int32_t *__restrict__ row_of_edge, const int32_t *__restrict__ rowptr_new,
+                              const int32_t *__restrict__ perm, const int32_t *__restrict__ in_rowptr,
+                              const int32_t *__restrict__ in_colidx, const int32_t *__restrict__ inv, int64_t E,
+                              int32_t *__restrict__ colidx_new) {
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < E; e += 4 * step) {
+        int32_t n[4], c[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) n[k] = e + k * step < E ? __ldg(row_of_edge + e + k * step) : -1;
+        int64_t pos[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            pos[k] = n[k] >= 0 ? (int64_t)__ldg(in_rowptr + __ldg(perm + n[k])) + (e + k * step - __ldg(rowptr_new + n[k])) : 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) c[k] = n[k] >= 0 ? __ldg(in_colidx + pos[k]) : 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (n[k] >= 0) colidx_new[e + k * step] = __ldg(inv + c[k]);
     }
 }
 

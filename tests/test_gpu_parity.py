@@ -935,3 +935,20 @@ def test_blocked_bfs_merge_by_slices_of_every_length(T, B, k):
     for s in gg.sources(g, 2, seed=3):
         lv = T.bfs_pull(G, P, s, tocab_threshold=0.0).cpu().numpy()
         assert np.array_equal(lv, oracle.bfs(g.V, rp, ci, s))
+
+
+@pytest.mark.parametrize("E", [1, 3, 4, 5, 9, 4099])
+def test_columns_outside_the_graph_are_refused_wherever_they_stand(T, E):
+    """Columns are checked four at a time, the last ones one by one."""
+    V = 100
+    rowptr = torch.full((V + 1,), E, dtype=torch.int32)
+    rowptr[0] = 0
+    good = torch.full((E,), V - 1, dtype=torch.int32)
+    assert T.graph_load_csr(rowptr.cuda(), good.cuda(), V=V).E == E
+    for at in sorted({0, 1, E // 2, E - 2, E - 1} & set(range(E))):
+        for c in (-1, V, 2 ** 31 - 1, -2 ** 31):
+            ci = good.clone()
+            ci[at] = c
+            with pytest.raises(T.TocabError) as e:
+                T.graph_load_csr(rowptr.cuda(), ci.cuda(), V=V)
+            assert e.value.status == -2
