@@ -180,10 +180,11 @@ __global__ void __launch_bounds__(BFS_THREADS, 8) k_bfs_block_level(const int32_
 //   else   : a lane per row with early exit (scan_rows).  Streaming here too, with an edge's row from the
 //            count of rows started up to it, was bound by its instructions: 385 against 363 us on the
 //            level with the largest frontier with cold caches, and slower still with warm ones.
-// Bound by reading the edges when it streams; k_bfs_block_level walks a row per lane there and waits
-// on one uncoalesced load and one random bitmap read at a time.  Two searches on a symmetrised R-MAT of
-// 5M vertices, 8 blocks, every level blocked: 5,781 us with that kernel alone (1,018 us for each of the
-// first two levels), 2,770 us with this one in the levels above the line at its launch.
+// Bound by reading the edges when it streams, by its instructions else (60% of issue slots); a lane per row
+// waits for uncoalesced loads and random bitmap reads there.  Two searches on a symmetrised R-MAT of 5M
+// vertices, 8 blocks, every level blocked: 5,781 us with k_bfs_block_level alone, then still an edge at a
+// time (1,018 us for each of the first two levels), 2,770 us with this one in the levels above the line at its
+// launch, 2,106 us with rows loaded a group ahead and scanned in steps and the merge as below.
 constexpr int BLK_THREADS = 1024;
 constexpr int BLK_CHUNK = 8192;  // rows: 8 groups per warp
 constexpr size_t BLK_MAX_SMEM = 104 * 1024;  // slices of up to 851,968 sources: two CTAs per SM

@@ -165,7 +165,7 @@ int launch_push_smem(const tc_part *p, const float *contrib, void *sums, const f
 // arrive finishes the range (and zeroes its sums again).
 //
 // What bounds it: the L1 requests for the contributions of distinct sources (some 15 lines per 32 edges
-// at R-MAT skew; L1 84% busy), next to one shared atomic per edge.  Wider ranges mean fewer distinct
+// at R-MAT skew; L1 68%, L2 59% busy), next to one shared atomic per edge.  Wider ranges mean fewer distinct
 // sources, but the lines of requests in flight need L1 too, so two CTAs of 1024 threads share an SM with at
 // most CUT_WIDTH * 8 bytes each.  Lanes take consecutive edges: four per lane as one wide load spread a
 // warp's sources over four times the lines (204 against 184 us per iteration).
