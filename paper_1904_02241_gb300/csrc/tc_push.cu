@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "tc_common_dev.cuh"
+#include "tc_walk.cuh"
 
 namespace tc {
 
@@ -208,27 +209,28 @@ __global__ void __launch_bounds__(PS_THREADS, 2) k_push_cut(const int4 *__restri
     const float scalef = *a.fx_scale * 0x1p-6f;  // |sum| < 2^55
     __syncthreads();
     // a lane's edges are 32 apart: consecutive edges, whose sources are close, share a load
-    int32_t i = t.y + (int32_t)threadIdx.x;
-    for (; t.z - i > 3 * PS_THREADS; i += 4 * PS_THREADS) {
-        int32_t sv[4];
-        uint32_t dv[4];
-        float cv[4];
+    walk_batched<4, PS_THREADS>(
+        (uint32_t)t.y + threadIdx.x, (uint32_t)t.z,
+        [&](uint32_t i) {
+            int32_t sv[4];
+            uint32_t dv[4];
+            float cv[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            sv[k] = ld_stream(src + i + k * PS_THREADS);
-            dv[k] = ld_stream(dst + i + k * PS_THREADS);
-        }
+            for (int k = 0; k < 4; ++k) {
+                sv[k] = ld_stream(src + i + k * PS_THREADS);
+                dv[k] = ld_stream(dst + i + k * PS_THREADS);
+            }
 #pragma unroll
-        for (int k = 0; k < 4; ++k) cv[k] = __ldg(a.contrib + sv[k]);
+            for (int k = 0; k < 4; ++k) cv[k] = __ldg(a.contrib + sv[k]);
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-            if (cv[k] != 0.0f) ps_add64(acc_lo + dv[k], acc_hi + dv[k], fx_round64(cv[k] * scalef));
-    }
-    for (; i < t.z; i += PS_THREADS) {
-        const uint32_t d = ld_stream(dst + i);
-        const float c = __ldg(a.contrib + ld_stream(src + i));
-        if (c != 0.0f) ps_add64(acc_lo + d, acc_hi + d, fx_round64(c * scalef));
-    }
+            for (int k = 0; k < 4; ++k)
+                if (cv[k] != 0.0f) ps_add64(acc_lo + dv[k], acc_hi + dv[k], fx_round64(cv[k] * scalef));
+        },
+        [&](uint32_t i) {
+            const uint32_t d = ld_stream(dst + i);
+            const float c = __ldg(a.contrib + ld_stream(src + i));
+            if (c != 0.0f) ps_add64(acc_lo + d, acc_hi + d, fx_round64(c * scalef));
+        });
     __syncthreads();
     const bool shared_range = t.w > 1;
     if (shared_range) {

@@ -1,0 +1,23 @@
+// Strided walks over edge positions.  A graph may have 2^31 - 2 edges, so a signed 32-bit position that
+// steps past the end of the last edges wraps to a negative one, below the end again.  These positions are
+// unsigned: a thread's last step leaves them below 2^32 as long as the batch is below 2^31.  Compiles as
+// plain C++ too, for the check of the positions on the host.
+#pragma once
+#include <stdint.h>
+
+#ifdef __CUDACC__
+#define TC_WALK __device__ __forceinline__
+#else
+#define TC_WALK inline
+#endif
+
+namespace tc {
+
+// batch(i) takes the positions i, i + STEP, ..., i + (N - 1) STEP, all below `end`; one(i) those left over.
+template <int N, int STEP, class Batch, class One>
+TC_WALK void walk_batched(uint32_t i, uint32_t end, Batch batch, One one) {
+    for (; i + (N - 1) * STEP < end; i += N * STEP) batch(i);
+    for (; i < end; i += STEP) one(i);
+}
+
+}  // namespace tc

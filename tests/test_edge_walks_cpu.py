@@ -1,0 +1,52 @@
+"""The kernels' walks over edge positions, compiled for the host: near the largest edge count every thread
+stays inside its edges and together they take each edge once."""
+import ctypes as C
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_1904_02241_gb300", "csrc")
+LAST = 2 ** 31 - 2   # the largest edge count that a graph may have
+
+SOURCE = r"""
+#include "tc_walk.cuh"
+// hits[i - first] counts position i; returns how many positions lay outside [first, end)
+extern "C" long batched(uint32_t first, uint32_t end, int threads, int32_t *hits) {
+    long off = 0;
+    auto one = [&](uint32_t i) {
+        if (i < first || i >= end) ++off; else ++hits[i - first];
+    };
+    for (int t = 0; t < threads && off == 0; ++t)
+        tc::walk_batched<4, 1024>(first + (uint32_t)t, end, [&](uint32_t i) { for (int k = 0; k < 4; ++k) one(i + k * 1024u); }, one);
+    return off;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def walks(tmp_path_factory):
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if cxx is None:
+        pytest.skip("no C++ compiler")
+    d = tmp_path_factory.mktemp("walks")
+    (d / "w.cpp").write_text(SOURCE)
+    subprocess.run([cxx, "-std=c++17", "-O1", "-shared", "-fPIC", "-I", CSRC, str(d / "w.cpp"), "-o", str(d / "w.so")],
+                   check=True)
+    return C.CDLL(str(d / "w.so"))
+
+
+def _all_taken_once(f, first, end, *args):
+    f.restype = C.c_long
+    hits = np.zeros(max(end - first, 1), np.int32)
+    off = f(C.c_uint32(first), C.c_uint32(end), *args, hits.ctypes.data_as(C.c_void_p))
+    assert off == 0 and np.all(hits[:end - first] == 1)
+
+
+@pytest.mark.parametrize("end", [LAST, LAST - 1, LAST - 1023, LAST - 4096, 5000, 4096, 1])
+@pytest.mark.parametrize("n", [0, 1, 1023, 1024, 1025, 3072, 3073, 4097, 9000])
+def test_push_tiles_stay_inside_their_edges(walks, end, n):
+    _all_taken_once(walks.batched, max(end - n, 0), end, C.c_int(1024))
