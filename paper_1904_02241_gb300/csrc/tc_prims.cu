@@ -6,6 +6,7 @@
 #include <mutex>
 
 #include "tc_internal.cuh"
+#include "tc_walk.cuh"
 
 namespace tc {
 
@@ -697,13 +698,13 @@ __global__ void __launch_bounds__(EXPAND_THREADS) k_expand_rows(const int32_t *_
                 __syncwarp();
                 const int32_t gend = __shfl_sync(0xffffffffu, e, 31 - __clz(rows));
                 int32_t started = 0;
-                for (; pos < gend; pos += 32) {
-                    const bool here = b < e && b >= pos && b - pos < 32;
-                    const unsigned starts = __reduce_or_sync(0xffffffffu, here ? 1u << (b - pos) : 0u);
-                    if (lane < gend - pos)
-                        row_of_edge[pos + lane] = list[started + __popc(starts & ((2u << lane) - 1u)) - 1];
+                walk<32>((uint32_t)pos, (uint32_t)gend, [&](uint32_t at) {
+                    const uint32_t d = (uint32_t)b - at;  // wraps above 32 for a row started before
+                    const unsigned starts = __reduce_or_sync(0xffffffffu, b < e && d < 32u ? 1u << d : 0u);
+                    if ((uint32_t)lane < (uint32_t)gend - at)
+                        row_of_edge[at + lane] = list[started + __popc(starts & ((2u << lane) - 1u)) - 1];
                     started += __popc(starts);
-                }
+                });
                 pos = gend;
                 __syncwarp();
             }

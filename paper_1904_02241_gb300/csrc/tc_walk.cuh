@@ -13,11 +13,17 @@
 
 namespace tc {
 
+// one(i) for the positions i, i + STEP, ... below `end`.
+template <int STEP, class One>
+TC_WALK void walk(uint32_t i, uint32_t end, One one) {
+    for (; i < end; i += STEP) one(i);
+}
+
 // batch(i) takes the positions i, i + STEP, ..., i + (N - 1) STEP, all below `end`; one(i) those left over.
 template <int N, int STEP, class Batch, class One>
 TC_WALK void walk_batched(uint32_t i, uint32_t end, Batch batch, One one) {
     for (; i + (N - 1) * STEP < end; i += N * STEP) batch(i);
-    for (; i < end; i += STEP) one(i);
+    walk<STEP>(i, end, one);
 }
 
 }  // namespace tc

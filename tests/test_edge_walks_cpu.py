@@ -24,6 +24,15 @@ extern "C" long batched(uint32_t first, uint32_t end, int threads, int32_t *hits
         tc::walk_batched<4, 1024>(first + (uint32_t)t, end, [&](uint32_t i) { for (int k = 0; k < 4; ++k) one(i + k * 1024u); }, one);
     return off;
 }
+// a warp's windows of 32 positions: a lane writes where it is below the end
+extern "C" long windows(uint32_t first, uint32_t end, int32_t *hits) {
+    long off = 0, n = 0;
+    tc::walk<32>(first, end, [&](uint32_t at) {
+        if (at < first || ++n > 1000) { ++off; return; }
+        for (uint32_t lane = 0; lane < 32; ++lane) if (lane < end - at) ++hits[at + lane - first];
+    });
+    return off;
+}
 """
 
 
@@ -50,3 +59,9 @@ def _all_taken_once(f, first, end, *args):
 @pytest.mark.parametrize("n", [0, 1, 1023, 1024, 1025, 3072, 3073, 4097, 9000])
 def test_push_tiles_stay_inside_their_edges(walks, end, n):
     _all_taken_once(walks.batched, max(end - n, 0), end, C.c_int(1024))
+
+
+@pytest.mark.parametrize("end", [LAST, LAST - 1, LAST - 31, LAST - 32, 2048, 1])
+@pytest.mark.parametrize("n", [0, 1, 31, 32, 33, 40, 2048])
+def test_row_ids_of_the_last_edges(walks, end, n):
+    _all_taken_once(walks.windows, max(end - n, 0), end)
