@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "tc_internal.cuh"
+#include "tc_walk.cuh"
 
 namespace tc {
 
@@ -190,6 +191,9 @@ __global__ void __launch_bounds__(SP_THREADS) k_spmv_merge(const float *__restri
 // product than with eight blocks (R-MAT 22: 1.7e-7 against 9.9e-8 in the 2-norm).
 constexpr int SPM_THREADS = 512;
 constexpr int64_t SPM_MIN_ENTRIES = 1 << 20;
+// Pieces are walked with signed 32-bit positions (with unsigned ones the walk past SPAN took R-MAT 23 in 16
+// blocks from 498 to 617 us), which a thread takes at most this far past the last piece.
+constexpr int SPM_PAST = 6 * SPM_THREADS;
 __device__ __forceinline__ void spm_add(float2 *acc, float v) {  // x: the sum, y: its error
     const float2 a = *acc;
     const float t = a.x + v;
@@ -308,6 +312,7 @@ static int build_staged(tc_part *p, tc_part *sp, const DeviceCaps &caps, cudaStr
     if (!pays) return fail(TC_ERR_UNSUPPORTED, "build_staged: too many pieces");
     TC_TRY(build_partition(p->g, TC_PUSH, nb, &pp, s, sp));
     if (sp->W > wmax || sp->W % 32 != 0 || !sp->id16.p || spm_smem_bytes(sp) > (size_t)caps.max_smem_optin) return fail(TC_ERR_UNSUPPORTED, "build_staged: width");
+    if (!fits_signed(sp->R, SPM_PAST)) return fail(TC_ERR_UNSUPPORTED, "build_staged: too many pieces");
     TC_TRY(build_tiles(sp, caps.sms, s));
     if (!sp->tiled) return fail(TC_ERR_UNSUPPORTED, "build_staged: no staged form");
     DevBuf iota, keys, perm, kt, vt, delta;

@@ -1,7 +1,7 @@
 // Strided walks over edge positions.  A graph may have 2^31 - 2 edges, so a signed 32-bit position that
-// steps past the end of the last edges wraps to a negative one, below the end again.  These positions are
-// unsigned: a thread's last step leaves them below 2^32 as long as the batch is below 2^31.  Compiles as
-// plain C++ too, for the check of the positions on the host.
+// steps past the end of the last edges wraps to a negative one, below the end again.  The walks' positions
+// are unsigned: a thread's last step leaves them below 2^32 as long as the batch is below 2^31.  Compiles
+// as plain C++ too, for the check of the positions on the host.
 #pragma once
 #include <stdint.h>
 
@@ -12,6 +12,9 @@
 #endif
 
 namespace tc {
+
+// Whether signed 32-bit positions of n items do not wrap when they go up to `past` beyond the end.
+constexpr bool fits_signed(int64_t n, int64_t past) { return n + past <= INT32_MAX; }
 
 // one(i) for the positions i, i + STEP, ... below `end`.
 template <int STEP, class One>

@@ -2,6 +2,7 @@
 stays inside its edges and together they take each edge once."""
 import ctypes as C
 import os
+import re
 import shutil
 import subprocess
 
@@ -33,6 +34,26 @@ extern "C" long windows(uint32_t first, uint32_t end, int32_t *hits) {
     });
     return off;
 }
+// a CTA's pieces of one block, with signed positions: the first `span` of a thread as loaded ahead, then the
+// others one by one
+extern "C" long pieces(uint32_t first, uint32_t end, int span, int32_t *hits) {
+    long off = 0, n = 0;
+    const int32_t r0 = (int32_t)first, r1 = (int32_t)end;
+    for (int32_t t = 0; t < 512 && off == 0; ++t) {
+        auto one = [&](int32_t r) {
+            if (r < r0 || r >= r1 || ++n > 100000) ++off; else ++hits[r - r0];
+        };
+        for (int h = 0; h < span; ++h)
+            if (r0 + t + h * 512 < r1) one(r0 + t + h * 512);
+        for (int32_t r = r0 + t + span * 512; r < r1 && off == 0; r += 512) one(r);
+    }
+    return off;
+}
+extern "C" int most_pieces(int past) {
+    int32_t n = INT32_MAX;
+    while (!tc::fits_signed(n, past)) --n;
+    return n;
+}
 """
 
 
@@ -43,7 +64,7 @@ def walks(tmp_path_factory):
         pytest.skip("no C++ compiler")
     d = tmp_path_factory.mktemp("walks")
     (d / "w.cpp").write_text(SOURCE)
-    subprocess.run([cxx, "-std=c++17", "-O1", "-shared", "-fPIC", "-I", CSRC, str(d / "w.cpp"), "-o", str(d / "w.so")],
+    subprocess.run([cxx, "-std=c++17", "-O1", "-fwrapv", "-shared", "-fPIC", "-I", CSRC, str(d / "w.cpp"), "-o", str(d / "w.so")],
                    check=True)
     return C.CDLL(str(d / "w.so"))
 
@@ -65,3 +86,20 @@ def test_push_tiles_stay_inside_their_edges(walks, end, n):
 @pytest.mark.parametrize("n", [0, 1, 31, 32, 33, 40, 2048])
 def test_row_ids_of_the_last_edges(walks, end, n):
     _all_taken_once(walks.windows, max(end - n, 0), end)
+
+
+def _constant(file, name):
+    text = open(os.path.join(CSRC, file)).read()
+    m = re.search(r"constexpr int " + name + r" = ([0-9]+)(?: \* SPM_THREADS)?;", text)
+    return int(m.group(1))
+
+
+@pytest.mark.parametrize("n", [0, 1, 511, 512, 513, 2049, 5000])
+@pytest.mark.parametrize("span", [1, 2, 4])
+def test_last_pieces_of_the_largest_staged_product(walks, n, span):
+    """Up to as many pieces as the staged product takes, its signed positions do not wrap."""
+    threads = _constant("tc_spmv.cu", "SPM_THREADS")
+    assert threads == 512
+    end = walks.most_pieces(C.c_int(_constant("tc_spmv.cu", "SPM_PAST") * threads))
+    assert end < LAST - span * threads
+    _all_taken_once(walks.pieces, end - n, end, C.c_int(span))
