@@ -33,6 +33,7 @@
 #include <vector>
 
 #include "tc_common_dev.cuh"
+#include "tc_walk.cuh"
 
 namespace tc {
 
@@ -355,7 +356,7 @@ __global__ void __launch_bounds__(BC_THREADS) k_bc_backward(const int32_t *__res
             e = rowptr[v + 1];
         }
         const bool small = e - s <= small_max;
-        double t = bc_group_sum<8>(bc_row_sum<4>(colidx, s + sub, small ? e : s, 8, coef_next));
+        double t = bc_group_sum<8>(bc_row_sum<4>(colidx, lane_first(s, e, sub), small ? e : s, 8, coef_next));
         unsigned wm = __ballot_sync(FULL_WARP, sub == 0 && !small && e - s <= hub_degree);
         while (wm) {
             const int l = __ffs(wm) - 1;

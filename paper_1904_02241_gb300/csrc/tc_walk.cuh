@@ -16,6 +16,10 @@ namespace tc {
 // Whether signed 32-bit positions of n items do not wrap when they go up to `past` beyond the end.
 constexpr bool fits_signed(int64_t n, int64_t past) { return n + past <= INT32_MAX; }
 
+// The first position of lane `lane` in [s, e): s + lane, or e if that is past the end (rows shorter than
+// the lanes that share them, where the sum could wrap).
+TC_WALK int32_t lane_first(int32_t s, int32_t e, int32_t lane) { return lane < e - s ? s + lane : e; }
+
 // one(i) for the positions i, i + STEP, ... below `end`.
 template <int STEP, class One>
 TC_WALK void walk(uint32_t i, uint32_t end, One one) {

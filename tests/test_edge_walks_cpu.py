@@ -49,6 +49,17 @@ extern "C" long pieces(uint32_t first, uint32_t end, int span, int32_t *hits) {
     }
     return off;
 }
+// eight lanes along one row, as far as 64-bit positions go on from each lane's first
+extern "C" long lanes(uint32_t first, uint32_t end, int32_t *hits) {
+    for (int lane = 0; lane < 8; ++lane) {
+        const int32_t at = tc::lane_first((int32_t)first, (int32_t)end, lane);
+        for (int64_t i = at; i < (int64_t)end; i += 8) {
+            if (i < (int64_t)first) return 1;
+            ++hits[i - first];
+        }
+    }
+    return 0;
+}
 extern "C" int most_pieces(int past) {
     int32_t n = INT32_MAX;
     while (!tc::fits_signed(n, past)) --n;
@@ -103,3 +114,9 @@ def test_last_pieces_of_the_largest_staged_product(walks, n, span):
     end = walks.most_pieces(C.c_int(_constant("tc_spmv.cu", "SPM_PAST") * threads))
     assert end < LAST - span * threads
     _all_taken_once(walks.pieces, end - n, end, C.c_int(span))
+
+
+@pytest.mark.parametrize("end", [LAST, LAST - 6, LAST - 7, 64])
+@pytest.mark.parametrize("n", [0, 1, 7, 8, 9, 64])
+def test_lanes_of_the_last_rows(walks, end, n):
+    _all_taken_once(walks.lanes, end - n, end)
