@@ -550,7 +550,9 @@ int tc_part_set_values(tc_part *p, const float *vals, int mem, void *stream);
  *   pieces are walked as one stream.
  *   p : a partition of the graph holding A, with values set by tc_part_set_values.
  *   x : float[V], y : float[V], device.
- * Asynchronous on `stream`.  Errors: TC_ERR_INVALID_ARG, TC_ERR_UNSUPPORTED, TC_ERR_CUDA.
+ * Asynchronous on `stream`.  With the finer cut, a device wait for a block of x that gives up (after
+ * about a second) makes that product NaN throughout; the next ones are not affected.
+ * Errors: TC_ERR_INVALID_ARG, TC_ERR_UNSUPPORTED, TC_ERR_CUDA.
  */
 int tc_spmv_tocab(const tc_part *p, const float *x, float *y, int mem, void *stream);
 

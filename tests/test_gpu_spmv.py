@@ -3,6 +3,9 @@ lane, then a 5-level shuffle tree), so row i may differ from the exact product b
 (d_i + 6) * 2^-24 * sum_k |a_ik x_k| (d_i = stored entries of the row): the standard bound for a
 summation whose longest chain has at most d_i + 5 roundings.  The inputs are the same FP32 values
 on both sides."""
+import ctypes as C
+import subprocess
+
 import numpy as np
 import pytest
 import torch
@@ -272,3 +275,32 @@ def test_staged_gc_pull_matches_oracle_within_the_fp32_bound(T, V, entries, B, s
     hit = np.zeros(V, dtype=bool)
     hit[np.repeat(np.arange(V), np.diff(rp))[ci == V // 5]] = True
     assert np.array_equal(~np.isfinite(T.spmv_tocab(P, xd).cpu().numpy()), hit)
+
+
+def test_a_wait_that_gave_up_spoils_no_later_product(T, tmp_path):
+    """The staged product's error flag, raised here from the host as a bounded wait that gives up raises
+    it, belongs to the product it was raised in: later ones, and products of new values, are right."""
+    from paper_1904_02241_gb300 import build
+    (tmp_path / "flag.cu").write_text('#include "tc_internal.cuh"\n'
+                                      'extern "C" int raise_flag(tc_part *p) {\n'
+                                      '    return p->sp ? (int)cudaMemset(p->sp_err.p, 1, 4) : -1;\n'
+                                      '}\n')
+    so = tmp_path / "flag.so"
+    subprocess.run([build.nvcc(), *build.NVCC_FLAGS, "-shared", str(tmp_path / "flag.cu"), "-o", str(so)], check=True)
+    raise_flag = C.CDLL(str(so)).raise_flag
+    raise_flag.argtypes = [C.c_void_p]
+    V, entries = 41344, 1 << 20
+    g = _big_matrix(V, entries, 3)
+    G = T.graph_load_csr(g.rowptr.cuda(), g.colidx.cuda(), V=V)
+    P = T.tocab_partition(G, T.TC_PUSH, 2)
+    vals = torch.from_numpy(np.random.default_rng(1).standard_normal(entries).astype(np.float32)).cuda()
+    x = torch.ones(V, device="cuda")
+    T.part_set_values(P, vals)
+    y = T.spmv_tocab(P, x)
+    torch.cuda.synchronize()
+    assert torch.isfinite(y).all()
+    assert raise_flag(P.handle) == 0
+    assert torch.equal(T.spmv_tocab(P, x), y)
+    assert raise_flag(P.handle) == 0
+    T.part_set_values(P, 2 * vals)
+    assert torch.equal(T.spmv_tocab(P, x), 2 * y)
