@@ -206,50 +206,69 @@ __device__ __forceinline__ unsigned long long fx_round64(float y) {
     return (b >> 31) ? (0ull - r) : r;
 }
 
-// The dangling mass of a push iteration in fixed point (`scalef` per unit).  A thread adds its vertices to
-// a DanglingSum; all threads of the CTA call finish(i): the CTA's sum goes to slot[i], and the last of n
-// arrivals adds the slots and writes D and D / V.  Integers: the same for any division of the vertices
-// among CTAs.  Ranks that are not finite (from initial ranks that are not) make D so too: they are added
-// as FP32 beside the sum, and their sum takes the slot, marked in bits that no sum of finite ranks
-// (below 2^56) has.
-struct DanglingSum {
-    static constexpr unsigned long long MARK = 0x4000000000000000ull;
+// The last CTA's part of DanglingSum, a call of its own: inlined, its FP64 arithmetic cost k_push_update the
+// registers of three CTAs per SM (46 instead of 32 per thread; R-MAT 22, 130 to 144 us).
+static __device__ __noinline__ void dangling_total(int32_t n, const unsigned long long *slot, const double *rest,
+                                                   unsigned *counter, float scalef, double *D, SpreadOut spread) {
+    __shared__ unsigned long long red5[32];
+    __shared__ double redd5[32];
+    __threadfence();
     unsigned long long t = 0;
-    float odd = 0.0f;  // sum of the ranks that are not finite
-    __device__ __forceinline__ void add(float r, float scalef) {
-        if (fabsf(r) <= 3.402823466e38f) t += fx_round64(r * scalef);
-        else odd += r;
+    double z = 0.0;
+    for (int32_t k = threadIdx.x; k < n; k += blockDim.x) {
+        t += __ldcg(slot + k);
+        const double x = __ldcg(rest + k);
+        if (__double_as_longlong(x) != 0ll) z += x;  // (an FP64 addition is slow here)
     }
-    __device__ __forceinline__ void finish(int32_t i, int32_t n, unsigned long long *slot, unsigned *counter,
-                                           float scalef, double *D, SpreadOut spread) {
+    t = block_sum<unsigned long long>(t, red5);
+    if (__syncthreads_or(__double_as_longlong(z) != 0ll)) z = block_sum<double>(z, redd5);
+    if (threadIdx.x == 0) {
+        const double d = (double)(long long)t / (double)scalef + z;
+        *D = d;
+        spread.write(d);
+        *counter = 0u;
+    }
+}
+
+// The dangling mass of a push iteration in fixed point (`scalef` per unit).  A thread adds its vertices to
+// a DanglingSum; all threads of the CTA call finish(i): the CTA's sum goes to slot[i] and rest[i], and the
+// last of n arrivals adds the slots and writes D and D / V.  Integers: the same for any division of the
+// vertices among CTAs.  What the fixed point does not hold is summed beside it in FP32, with the CTAs' sums
+// in FP64: ranks that are not finite, and the fractions of ranks below 2^-32 of the caller's L1 mass (the
+// ranks themselves below 2^-56 of it), which are all there is when the dangling vertices hold next to
+// nothing of a large mass.
+struct DanglingSum {
+    unsigned long long t = 0;
+    float odd = 0.0f;
+    __device__ __forceinline__ void add(float r, float scalef, float inv_scalef) {
+        const float y = r * scalef, a = fabsf(y);
+        if (a >= 0x1p23f && a < 0x1p62f) {  // a whole number: no rounding
+            const uint32_t b = __float_as_uint(y);
+            const unsigned long long u = (unsigned long long)((b & 0x7fffffu) | 0x800000u) << (((b >> 23) & 0xffu) - 150u);
+            t += (b >> 31) ? 0ull - u : u;
+        } else if (a < 0x1p23f) {
+            const int32_t u = __float2int_rn(y);
+            t += (unsigned long long)(long long)u;
+            odd += r - (float)u * inv_scalef;  // exact
+        } else {
+            odd += r;
+        }
+    }
+    __device__ __forceinline__ void finish(int32_t i, int32_t n, unsigned long long *slot, double *rest,
+                                           unsigned *counter, float scalef, double *D, SpreadOut spread) {
         __shared__ bool am_last4;
         __shared__ unsigned long long red4[32];
         __shared__ float redf4[32];
         t = block_sum<unsigned long long>(t, red4);
-        if (__syncthreads_or(odd != 0.0f)) t = MARK | __float_as_uint(block_sum<float>(odd, redf4));
+        if (__syncthreads_or(odd != 0.0f)) odd = block_sum<float>(odd, redf4);
         if (threadIdx.x == 0) {
             slot[i] = t;
+            rest[i] = (double)odd;
             __threadfence();
             am_last4 = atomicAdd(counter, 1u) == (unsigned)n - 1u;
         }
         __syncthreads();
-        if (!am_last4) return;
-        __threadfence();
-        t = 0;
-        odd = 0.0f;
-        for (int32_t k = threadIdx.x; k < n; k += blockDim.x) {
-            const unsigned long long x = __ldcg(slot + k);
-            if ((x >> 56) == (MARK >> 56)) odd += __uint_as_float((uint32_t)x);
-            else t += x;
-        }
-        t = block_sum<unsigned long long>(t, red4);
-        odd = block_sum<float>(odd, redf4);
-        if (threadIdx.x == 0) {
-            const double d = (double)(long long)t / (double)scalef + (double)odd;
-            *D = d;
-            spread.write(d);
-            *counter = 0u;
-        }
+        if (am_last4) dangling_total(n, slot, rest, counter, scalef, D, spread);
     }
 };
 
@@ -326,6 +345,7 @@ struct PushCutArgs {
     unsigned long long *sums;     // zero between launches; ranges of several tiles meet there
     int32_t *range_count;
     unsigned long long *dslot;    // [B]
+    double *drest;                // [B]
     unsigned *counter;
 };
 int launch_push_cut(const tc_part *p, PushCutArgs a, cudaStream_t s);

@@ -23,6 +23,7 @@ struct UpdateArgs {
     const float *S_cur;     // D / V of *D_cur and of *D_next in FP32
     float *S_next;
     double *dpart;          // per-CTA partial dangling sums
+    double *drest;          // ... and of what fixed point does not hold (push)
     unsigned *counter;      // arrival counter for the last-CTA reduction
     const float *inv_outdeg;
     float *rank_out;        // may be null (only the last iteration writes ranks)
@@ -822,11 +823,11 @@ __global__ void __launch_bounds__(PR_THREADS) k_push_update(void *sums, UpdateAr
             *sp = 0.0f;
         }
         const float d = apply_update(u, (int32_t)v, s, spread);
-        if (FIXED) dfix.add(d, push_scale(u.fx_scale));
-        else dsum += d;
+        if (!FIXED) dsum += d;
+        else if (d != 0.0f) dfix.add(d, push_scale(u.fx_scale), inv_scalef);
     }
     if (FIXED) {
-        dfix.finish(blockIdx.x, gridDim.x, reinterpret_cast<unsigned long long *>(u.dpart), u.counter,
+        dfix.finish(blockIdx.x, gridDim.x, reinterpret_cast<unsigned long long *>(u.dpart), u.drest, u.counter,
                     push_scale(u.fx_scale), u.D_next, spread_out(u));
         return;
     }
@@ -1059,6 +1060,7 @@ static int pagerank_impl(const tc_graph *cg, const tc_part *part, const tc_pr_pa
     u.drop = pp->dangling == TC_DANGLING_DROP;
     u.V = V;
     u.dpart = st.dpart;
+    u.drest = st.dpart + st.dpart_cap;
     u.counter = st.counter;
     const bool renumbered = part && part->order == TC_ORDER_OUTDEGREE;
     u.inv_outdeg = renumbered ? part->inv_outdeg.as<float>() : g->inv_outdeg.as<float>();
@@ -1144,6 +1146,7 @@ static int pagerank_impl(const tc_graph *cg, const tc_part *part, const tc_pr_pa
                 a.fx_scale = st.scale;
                 a.sums = reinterpret_cast<unsigned long long *>(st.sums);
                 a.dslot = reinterpret_cast<unsigned long long *>(st.dpart);
+                a.drest = st.dpart + st.dpart_cap;
                 a.counter = st.counter;
                 TC_TRY(launch_push_cut(part, a, s));
             } else if (push_staged)

@@ -261,9 +261,9 @@ __global__ void __launch_bounds__(PS_THREADS, 2) k_push_cut(const int4 *__restri
         if (a.rank_out) a.rank_out[lo + v] = r;
         const float inv = __ldg(a.inv_outdeg + lo + v);
         a.contrib_next[lo + v] = r * inv;
-        if (inv == 0.0f) dangling.add(r, scalef);
+        if (inv == 0.0f) dangling.add(r, scalef, inv_scalef);
     }
-    dangling.finish(t.x, a.B, a.dslot, a.counter, scalef, a.D_next, a.spread);
+    dangling.finish(t.x, a.B, a.dslot, a.drest, a.counter, scalef, a.D_next, a.spread);
 }
 
 // First edge of every range (keys ascending by range, n of them), b in [0, B].

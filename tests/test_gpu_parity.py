@@ -952,3 +952,27 @@ def test_columns_outside_the_graph_are_refused_wherever_they_stand(T, E):
             with pytest.raises(T.TocabError) as e:
                 T.graph_load_csr(rowptr.cuda(), ci.cuda(), V=V)
             assert e.value.status == -2
+
+
+@pytest.mark.parametrize("total,damping", [(1.0, 0.85), (2.0 ** 20, 0.85), (2.0 ** 45, 0.85), (2.0 ** 100, 0.85),
+                                           (2.0 ** -60, 1.0)])
+def test_push_dangling_mass_far_below_the_total(T, total, damping):
+    """Two vertices that rank each other hold nearly all of the caller's mass; the dangling vertices hold
+    ranks around 1 (2^-66 where there is no teleport), which every vertex without in-edges must see.  The mass is summed in FP32
+    per CTA: a thread's vertices here are at most three and the block's tree has ten levels, an iteration
+    adds four roundings, so four iterations stay below 4 * 17 roundings of 2^-24, 4.1e-6."""
+    V, small = 3000, 1.0 if damping < 1 else 2.0 ** -66
+    rng = np.random.default_rng(4)
+    edges = [(0, 1), (1, 0)] + [(v, 0) for v in range(V // 2, V)]  # 2 .. V/2 - 1 are dangling
+    g = gg.from_edge_list(V, edges)
+    G = _load(T, g)
+    rp, ci = g.numpy()
+    init = torch.tensor(small * rng.uniform(1, 2, V), dtype=torch.float32)
+    init[:2] = total / 2
+    alone = np.arange(2, V)  # no in-edges
+    P = T.tocab_partition(G, T.TC_PUSH, 2)
+    for part, lb in ((P, 0), (P, 8), (None, 0)):
+        for iters in (4, 1, 2, 3):
+            r = T.pagerank_push(G, part, damping=damping, iters=iters, init=init.cuda(), lb_warp_min=lb).cpu().numpy()
+            want = oracle.pagerank_push(V, rp, ci, damping=damping, iters=iters, init=init.double().numpy())
+            np.testing.assert_allclose(r[alone], want[alone], rtol=4.1e-6, atol=0)
