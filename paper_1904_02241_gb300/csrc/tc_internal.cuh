@@ -16,6 +16,14 @@ namespace tc {
 void set_error(const char *fmt, ...);
 int fail(int status, const char *fmt, ...);   // sets last error, returns status
 
+// The calling thread's error message as it stands, put back by restore(): for a step whose failure is not
+// the call's (the call goes on another way and returns TC_OK, which leaves the message alone).
+struct KeptError {
+    char text[1024];
+    KeptError();
+    void restore() const;
+};
+
 #define TC_CUDA(call)                                                                   \
     do {                                                                                \
         cudaError_t err__ = (call);                                                     \

@@ -135,7 +135,7 @@ void cache_free(void *p, size_t bytes, int device) {
     if (cur >= 0) cudaSetDevice(cur);
 }
 
-static thread_local char g_last_error[1024] = "";
+static thread_local char g_last_error[sizeof(KeptError::text)] = "";
 
 void set_error(const char *fmt, ...) {
     va_list ap;
@@ -151,6 +151,9 @@ int fail(int status, const char *fmt, ...) {
     va_end(ap);
     return status;
 }
+
+KeptError::KeptError() { memcpy(text, g_last_error, sizeof(text)); }
+void KeptError::restore() const { memcpy(g_last_error, text, sizeof(text)); }
 
 int device_caps(DeviceCaps *caps) {
     TC_CUDA(cudaGetDevice(&caps->device));

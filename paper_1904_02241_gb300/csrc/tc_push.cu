@@ -346,11 +346,14 @@ int ensure_push_cut(tc_part *p, cudaStream_t s) {
         return TC_OK;
     }
     p->cut_tried = true;
+    const KeptError kept;
     const int st = build_push_cut(p, s);
     if (st == TC_OK) return TC_OK;
     cudaStreamSynchronize(s);
     for (DevBuf *d : {&p->cut_src, &p->cut_dst, &p->cut_count, &p->cut_tiles}) d->release();
-    return st == TC_ERR_OOM ? TC_OK : st;
+    if (st != TC_ERR_OOM) return st;
+    kept.restore();
+    return TC_OK;
 }
 
 int launch_push_cut(const tc_part *p, PushCutArgs a, cudaStream_t s) {

@@ -410,6 +410,7 @@ extern "C" int tc_part_set_values(tc_part *p, const float *vals, int mem, void *
         p->sp_tried = true;
         tc_part *sp = new (std::nothrow) tc_part();
         if (sp) {
+            const KeptError kept;
             const int st = build_staged(p, sp, caps, s);
             if (st == TC_OK) {
                 p->sp = sp;
@@ -419,6 +420,7 @@ extern "C" int tc_part_set_values(tc_part *p, const float *vals, int mem, void *
                 p->sp_perm.release();
                 p->sp_vals.release();
                 if (st != TC_ERR_OOM && st != TC_ERR_UNSUPPORTED) return st;
+                kept.restore();
             }
         }
     }

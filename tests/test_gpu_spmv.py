@@ -304,3 +304,23 @@ def test_a_wait_that_gave_up_spoils_no_later_product(T, tmp_path):
     assert raise_flag(P.handle) == 0
     T.part_set_values(P, 2 * vals)
     assert torch.equal(T.spmv_tocab(P, x), 2 * y)
+
+
+def test_declining_the_staged_form_leaves_the_error_message_alone(T):
+    """A uniform matrix in one block, whose finer cut would have too many pieces: the values are set the
+    general way, the call succeeds, and the thread's message stays that of its last failed call."""
+    V = 1000000
+    gen = torch.Generator(device="cuda").manual_seed(2)
+    key = torch.unique(torch.randint(V * V, (6 * V,), generator=gen, device="cuda"))
+    deg = torch.bincount(key // V, minlength=V)
+    rowptr = torch.cat([deg.new_zeros(1), torch.cumsum(deg, 0)]).to(torch.int32)
+    G = T.graph_load_csr(rowptr, (key % V).to(torch.int32), V=V)
+    P = T.tocab_partition(G, T.TC_PUSH, 1)
+    with pytest.raises(T.TocabError):
+        T.graph_load_csr(torch.tensor([1, 1], dtype=torch.int32), torch.zeros(1, dtype=torch.int32), V=1)
+    before = T.lib().tc_last_error()
+    assert before
+    T.part_set_values(P, torch.ones(G.E, device="cuda"))
+    y = T.spmv_tocab(P, torch.ones(V, device="cuda"))
+    assert T.lib().tc_last_error() == before
+    assert torch.equal(y, deg.float())
