@@ -242,8 +242,9 @@ struct tc_part {
     tc::DevBuf sp_perm, sp_vals, sp_err;
     int32_t nptiles = 0;        // push, W * 8 bytes within shared memory: tiles of the staged push
     // push: the edges by destination range of cut_W vertices (fixed-point staged push; tc_push.cu),
-    // built on first use
+    // built when push calls have asked for enough iterations
     bool cut_tried = false;
+    int64_t push_iters = 0;     // iterations asked for so far, while there is no cut
     int32_t smem_stage = 0;     // as asked for: < 0 never staged
     int32_t cut_W = 0, cut_B = 0, cut_ntiles = 0;
     tc::DevBuf cut_src;         // int32[E]: source
@@ -293,7 +294,7 @@ int32_t tile_max_width(int max_smem_optin);
 // Staged push (tc_push.cu): widest destination range in shared memory, its tiles, the scatter.
 int32_t push_smem_width(int max_smem_optin);
 int build_push_tiles(tc_part *p, int sms, cudaStream_t s);
-int ensure_push_cut(tc_part *p, cudaStream_t s);
+int ensure_push_cut(tc_part *p, int32_t iters, cudaStream_t s);
 int launch_push_smem(const tc_part *p, const float *contrib, void *sums, const float *fx_scale, bool fixed,
                      cudaStream_t s);
 int build_tiles(tc_part *p, int sms, cudaStream_t s);

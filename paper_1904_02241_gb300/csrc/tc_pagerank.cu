@@ -1026,7 +1026,7 @@ static int pagerank_impl(const tc_graph *cg, const tc_part *part, const tc_pr_pa
     // or a per-block table) is given, a partition's scatter goes by destination ranges, else edge-parallel
     const bool push_fixed = pp->merge_mode != TC_PUSH_FLOAT;
     const bool push_whole = push && pp->lb_warp_min == 0 && !(part && part->lb_tab.p);  // no TWC threshold
-    if (push_whole && part && push_fixed) TC_TRY(ensure_push_cut(const_cast<tc_part *>(part), s));
+    if (push_whole && part && push_fixed) TC_TRY(ensure_push_cut(const_cast<tc_part *>(part), pp->iters, s));
     const bool push_cut = push_whole && part && push_fixed && part->cut_ntiles > 0;
     if (push_cut && part->cut_B > max_ctas) max_ctas = part->cut_B;  // one dangling slot per range
     if (part && !push && part->nranges > max_ctas) max_ctas = part->nranges;  // one dangling slot per range

@@ -976,3 +976,33 @@ def test_push_dangling_mass_far_below_the_total(T, total, damping):
             r = T.pagerank_push(G, part, damping=damping, iters=iters, init=init.cuda(), lb_warp_min=lb).cpu().numpy()
             want = oracle.pagerank_push(V, rp, ci, damping=damping, iters=iters, init=init.double().numpy())
             np.testing.assert_allclose(r[alone], want[alone], rtol=4.1e-6, atol=0)
+
+
+def test_push_builds_its_destination_ranges_when_they_pay(T):
+    """A partition asked for fewer than three iterations keeps the edges it has; the call that brings them
+    to three takes 6 B per edge more.  The ranks are the same bits throughout."""
+    V, m = 1 << 17, 4000000
+    rng = np.random.default_rng(6)
+    g = gg.from_edge_list(V, rng.integers(0, V, (m, 2)))
+    G = _load(T, g)
+
+    def used():
+        torch.cuda.synchronize()
+        T.set_device_memory_limit(1 << 50)  # returns the cached blocks
+        T.set_device_memory_limit(0)
+        return T.device_memory_held()
+
+    want = {n: T.pagerank_push(G, None, iters=n) for n in (0, 1, 5)}
+    P = T.tocab_partition(G, T.TC_PUSH, 3)
+    T.pagerank_push(G, P, iters=1, lb_warp_min=8)  # the scatter's own scratch
+    before = used()
+    for n in (0, 1, 0, 1, 0):
+        assert torch.equal(T.pagerank_push(G, P, iters=n), want[n])
+        assert used() == before
+    assert torch.equal(T.pagerank_push(G, P, iters=1), want[1])
+    assert before + 6 * g.E <= used() < before + 6 * g.E + (1 << 20)
+    assert torch.equal(T.pagerank_push(G, P, iters=5), want[5])
+    Q = T.tocab_partition(G, T.TC_PUSH, 3)
+    held = used()
+    assert torch.equal(T.pagerank_push(G, Q, iters=5), want[5])
+    assert used() >= held + 6 * g.E
