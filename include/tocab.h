@@ -149,7 +149,9 @@ typedef struct tc_part_params {
                                  shared memory (W * 8 bytes, about 29K vertices; the
                                  TC_BLOCKS_SMEM policy picks that width) and accumulate FP32
                                  sums there too; fixed-point sums go through ranges of the
-                                 library's own unless -1 (then always the global scatters) */
+                                 library's own, and tc_part_set_values may keep a finer cut,
+                                 unless -1 (then always the global scatters and the general
+                                 SpMV) */
     int32_t vertex_order;     /* pull only: TC_ORDER_NATURAL (0) or TC_ORDER_OUTDEGREE (1), below */
     int32_t direct_blocks;    /* renumbered pull only: local rows with a single edge whose source
                                  lies in the first `direct_blocks` blocks leave the blocked CSR
@@ -534,9 +536,11 @@ int tc_spmv(const tc_graph *g, const float *vals, const float *x, float *y, int 
  * column) pieces (GC-push SpMV).  The partition keeps the values in its own entry order (the
  * first call also records that order: the partition's stable sorts again, carrying entry
  * positions).  From 2^20 entries on a TC_PUSH partition may keep them in a finer cut instead, whose
- * blocks of x fit one CTA's shared memory (built by the first call; not under a memory limit, nor
- * where its memory is not to be had or its pieces would cost more than it gains).  For the SpMV of
- * Sec. 4.  Synchronises.
+ * blocks of x fit one CTA's shared memory (built by the first call; not with smem_stage = -1 or under
+ * a memory limit, nor where its memory is not to be had or its pieces would cost more than it gains).
+ * The first call takes longer with it and each product less: R-MAT 22 in 8 blocks, 2.9 against
+ * 0.7 ms, then 254 against 407 us, so it pays from 15 products on (other matrices 17 to 38); smem_stage = -1 declines it.
+ * For the SpMV of Sec. 4.  Synchronises.
  * Errors: TC_ERR_INVALID_ARG (NULL), TC_ERR_UNSUPPORTED (host values, a renumbered partition),
  * TC_ERR_OOM, TC_ERR_CUDA.
  */

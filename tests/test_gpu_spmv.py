@@ -324,3 +324,36 @@ def test_declining_the_staged_form_leaves_the_error_message_alone(T):
     y = T.spmv_tocab(P, torch.ones(V, device="cuda"))
     assert T.lib().tc_last_error() == before
     assert torch.equal(y, deg.float())
+
+
+def test_smem_stage_declines_the_staged_form(T):
+    """smem_stage = -1: the general form, as under a memory limit (the same bits), and none of the staged
+    form's memory."""
+    V, entries = 41344, 1 << 20
+    g = _big_matrix(V, entries, 3)
+    G = T.graph_load_csr(g.rowptr.cuda(), g.colidx.cuda(), V=V)
+    rng = np.random.default_rng(1)
+    vals = torch.from_numpy(rng.standard_normal(entries).astype(np.float32)).cuda()
+    x = torch.from_numpy(rng.standard_normal(V).astype(np.float32)).cuda()
+
+    def used():
+        torch.cuda.synchronize()
+        T.set_device_memory_limit(1 << 50)  # returns the cached blocks
+        T.set_device_memory_limit(0)
+        return T.device_memory_held()
+
+    def product(limit, **kw):
+        P = T.tocab_partition(G, T.TC_PUSH, 2, **kw)
+        before = used()
+        T.set_device_memory_limit(limit)
+        try:
+            T.part_set_values(P, vals)
+        finally:
+            T.set_device_memory_limit(0)
+        return T.spmv_tocab(P, x), used() - before
+
+    general, size = product(1 << 40)
+    declined, size_declined = product(0, smem_stage=-1)
+    assert torch.equal(declined, general) and size_declined == size
+    _, size_staged = product(0)
+    assert size_staged > size
