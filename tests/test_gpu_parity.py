@@ -1006,3 +1006,34 @@ def test_push_builds_its_destination_ranges_when_they_pay(T):
     held = used()
     assert torch.equal(T.pagerank_push(G, Q, iters=5), want[5])
     assert used() >= held + 6 * g.E
+
+
+@pytest.mark.parametrize("V,B", [(4097, 1), (20000, 3), (60001, 5)])
+@pytest.mark.parametrize("sums", ["fixed", "float"])
+def test_push_staged_by_the_partitions_blocks_under_a_memory_limit(T, V, B, sums):
+    """At a memory limit of what is held there are no destination ranges: smem_stage = 1 scatters into the
+    shared sums of the partition's own blocks.  Fixed-point sums are the row scatter's bits, with ranks of
+    either sign (carries between the halves of a sum) and a vertex that half the edges enter (several
+    tiles); FP32 sums are the oracle's ranks."""
+    rng = np.random.default_rng(V)
+    e = np.stack([rng.integers(0, V, 14 * V), rng.integers(0, V, 14 * V)], axis=1)
+    e[: 7 * V, 1] = V // 3
+    g = gg.from_edge_list(V, e)
+    G = _load(T, g)
+    init = torch.tensor(rng.standard_normal(V) / V, dtype=torch.float32)
+    P = T.tocab_partition(G, T.TC_PUSH, B, smem_stage=1)
+    kw = dict(iters=3, init=init.cuda())
+    want = T.pagerank_push(G, P, lb_warp_min=8, **kw)  # sizes the scratch too
+    held = T.device_memory_held()
+    T.set_device_memory_limit(1)  # returns the cached blocks
+    try:
+        assert T.device_memory_held() <= held
+        r = T.pagerank_push(G, P, sums=sums, **kw)
+    finally:
+        T.set_device_memory_limit(0)
+    if sums == "fixed":
+        assert torch.equal(r, want)
+        assert torch.equal(T.pagerank_push(G, P, **kw), want)  # by destination ranges now
+    rp, ci = g.numpy()
+    ora = oracle.pagerank_push(V, rp, ci, iters=3, init=init.double().numpy())
+    assert np.abs(r.cpu().numpy() - ora).sum() <= 1e-5 * np.abs(ora).sum()
