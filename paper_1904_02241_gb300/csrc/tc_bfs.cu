@@ -188,6 +188,10 @@ __global__ void __launch_bounds__(BFS_THREADS, 8) k_bfs_block_level(const int32_
 constexpr int BLK_THREADS = 1024;
 constexpr int BLK_CHUNK = 8192;  // rows: 8 groups per warp
 constexpr size_t BLK_MAX_SMEM = 104 * 1024;  // slices of up to 851,968 sources: two CTAs per SM
+// Below, a level has too few chunks to fill the chip and the slices' loads show.  Two searches on symmetrised
+// graphs, 8 blocks, without and with this kernel: R-MAT of 1.8M edges 463 and 606 us, 7.6M 581 and 606, 15M 677
+// and 702, 31M 1,172 and 939; uniform 8M 593 and 628, 17M 904 and 907, 34M 1,346 and 1,287.
+constexpr int64_t BLK_MIN_EDGES = 1 << 24;
 
 // Bit test of column c against the slice that starts at column lo (a multiple of 32).
 __device__ __forceinline__ bool in_slice(const uint32_t *sl, int32_t c, int32_t lo) {
@@ -922,7 +926,7 @@ static int bfs_impl(const tc_graph *cg, const tc_part *part, int32_t source, con
     // blocked levels with the slice in shared memory: two CTAs per SM
     int blk_grid = 0;
     const size_t blk_smem = part ? (size_t)(part->W / 32) * 4 : 0;
-    if (part && bp->tocab_threshold >= 0.0f && part->R > 0 && part->W % 32 == 0 && blk_smem <= BLK_MAX_SMEM) {
+    if (part && g->E >= BLK_MIN_EDGES && bp->tocab_threshold >= 0.0f && part->R > 0 && part->W % 32 == 0 && blk_smem <= BLK_MAX_SMEM) {
         TC_CUDA(cudaFuncSetAttribute(k_bfs_block_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BLK_MAX_SMEM));
         const int64_t chunks = (part->R + BLK_CHUNK - 1) / BLK_CHUNK;
         blk_grid = (int)(chunks < 2 * caps.sms ? chunks : 2 * caps.sms);

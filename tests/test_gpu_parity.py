@@ -1037,3 +1037,35 @@ def test_push_staged_by_the_partitions_blocks_under_a_memory_limit(T, V, B, sums
     rp, ci = g.numpy()
     ora = oracle.pagerank_push(V, rp, ci, iters=3, init=init.double().numpy())
     assert np.abs(r.cpu().numpy() - ora).sum() <= 1e-5 * np.abs(ora).sum()
+
+
+@pytest.fixture(scope="module")
+def large_symmetric():
+    """Symmetric graphs of 2^24 edges and more: R-MAT, uniform, and one whose middle third of the vertices
+    never holds a frontier vertex."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    a = gg.symmetrize(gg.rmat(19, device="cuda"))
+    V, deg = a.V, (a.rowptr[1:] - a.rowptr[:-1]).long()
+    row = torch.cat([deg, deg.new_zeros(V), deg])
+    islands = gg.CSRGraph(3 * V, torch.cat([row.new_zeros(1), torch.cumsum(row, 0)]).to(torch.int32),
+                          torch.cat([a.colidx, a.colidx + 2 * V]), "islands")
+    return {"rmat": gg.symmetrize(gg.rmat(20, device="cuda")), "islands": islands,
+            "er": gg.symmetrize(gg.erdos_renyi(700001, 9 * 10 ** 6, seed=8, device="cuda"))}
+
+
+@pytest.mark.parametrize("name,B", [("rmat", 2), ("rmat", 3), ("rmat", 8), ("rmat", 100), ("er", 1), ("er", 7),
+                                    ("islands", 5), ("islands", 150)])
+def test_large_blocked_bfs_levels_from_shared_memory(T, large_symmetric, name, B):
+    """From 2^24 edges on, blocked levels with most edges to scan keep the block's bitmap slice in shared
+    memory: chunks of 8,192 rows inside one block and across block ends, blocks without a frontier vertex,
+    streamed and early-exit levels."""
+    g = large_symmetric[name]
+    assert g.E >= 1 << 24
+    G = _load(T, g)
+    P = T.tocab_partition(G, T.TC_PULL, B, smem_stage=-1)
+    rp, ci = g.to("cpu").numpy()
+    for s in gg.sources(g.to("cpu"), 2, seed=41):
+        lv, st = T.bfs_pull(G, P, s, tocab_threshold=0.0, return_stats=True)
+        np.testing.assert_array_equal(lv.cpu().numpy(), oracle.bfs(g.V, rp, ci, s))
+        assert st.tocab_levels == st.levels
