@@ -300,6 +300,7 @@ int launch_push_smem(const tc_part *p, const float *contrib, void *sums, const f
 int build_tiles(tc_part *p, int sms, cudaStream_t s);
 size_t merge_smem_bytes(int32_t k, int32_t B);   // dynamic shared memory of the ordered pull merge
 size_t merge_atomic_smem_bytes(int32_t k, int32_t B, bool fixed);  // ... of the one-accumulator merges
+int32_t default_merge_range(int32_t V, int sms);   // width of the merge ranges when none is asked for
 // tc_tocab_partition's work on a fresh handle.
 int build_partition(const tc_graph *g, int dir, int32_t num_blocks, const tc_part_params *pp, cudaStream_t s,
                     tc_part *p);

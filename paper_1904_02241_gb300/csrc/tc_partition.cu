@@ -512,6 +512,13 @@ static int weighted_ranges(tc_part *p, int32_t kmax, cudaStream_t s, int grid) {
     return TC_OK;
 }
 
+// 8192 (longest slices that fit well), smaller for small graphs: >= 2 ranges per SM
+int32_t default_merge_range(int32_t V, int sms) {
+    int32_t k = 8192;
+    while (k > 1024 && ((int64_t)V + k - 1) / k < 2 * sms) k >>= 1;
+    return k;
+}
+
 int build_partition(const tc_graph *g, int dir, int32_t num_blocks, const tc_part_params *pp, cudaStream_t s,
                     tc_part *p) {
     DeviceCaps caps;
@@ -543,10 +550,8 @@ int build_partition(const tc_graph *g, int dir, int32_t num_blocks, const tc_par
     const float frac = (pp && pp->l2_fraction > 0) ? pp->l2_fraction : 0.0f;
     if (pp && pp->merge_range > 0) {
         p->k = pp->merge_range;
-    } else {  // 8192 (longest slices that fit well), smaller for small graphs: >= 2 ranges per SM
-        int64_t k = 8192;
-        while (k > 1024 && ((int64_t)V + k - 1) / k < 2 * caps.sms) k >>= 1;
-        p->k = (int32_t)k;
+    } else {
+        p->k = default_merge_range(V, caps.sms);
     }
     if (p->k % 32 != 0) return fail(TC_ERR_INVALID_ARG, "merge_range must be a multiple of 32");
     p->hub_degree = (pp && pp->hub_degree > 0) ? pp->hub_degree : 2048;

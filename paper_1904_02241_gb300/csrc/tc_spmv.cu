@@ -175,8 +175,8 @@ __global__ void __launch_bounds__(SP_THREADS) k_spmv_merge(const float *__restri
 }
 
 // Staged GC-pull.  With blocks of x that only fit the L2, an entry costs a random L2 request, and those
-// come at some 190 G/s whatever the order of the rows.  So from SPM_MIN_ENTRIES entries on (below, the
-// launches dominate either way), where it pays, the values get a finer cut of the matrix whose blocks of x
+// come at some 190 G/s whatever the order of the rows.  So from SPM_MIN_ENTRIES entries on (below, a product
+// gains 8 to 20 of 36 to 50 us, and setting the values takes some 500 us longer), where it pays, the values get a finer cut of the matrix whose blocks of x
 // fit one CTA's shared memory, in the staged form of the rank gather (tc_tile.cu) with a value per entry:
 // the entries stream at 6 B each and x is read in shared memory.
 // More pieces come with it, so their merge is a kernel of its own.  R-MAT 22, 8 blocks: 404 us the general
@@ -280,12 +280,17 @@ __global__ void __launch_bounds__(SP_THREADS) k_block_changes(const int32_t *__r
     if ((threadIdx.x & 31) == 0 && n) atomicAdd(count, (unsigned long long)n);
 }
 
-// Does the staged form pay?  Its gather is always the faster one, its merge has more pieces: where nearly
-// every entry becomes a piece and the loaded blocks have few of them, the merge takes what the gather gains.
-// Pieces beyond the loaded ones, of the entries, and times against the general form: uniform matrix of 16
-// entries per row, 4 blocks: 0.51 (1M rows) 101 against 136 us, 0.61 (2M) 188 / 206, 0.68 (4M) 370 / 354, 0.71
-// (8M) 736 / 694; with 16 blocks 0.33 (8M) 735 / 840; R-MAT 22 with 8 blocks below 0.4, 245 / 404.
-static int staged_pays(const tc_part *p, int32_t W, const DeviceCaps &caps, cudaStream_t s, bool *pays) {
+// Does the staged form pay, with nb blocks of W columns?  Its gather is always the faster one, its merge has
+// more pieces in more slices (a piece costs a random read and write of shared memory, a slice of a block and
+// range a barrier), and takes what the gather gains where rows are short.  The line was fitted to 544 uniform
+// and R-MAT matrices of 150K to 8M rows, 2 to 64 entries per row, 1 to 32 loaded blocks: of the 360 it takes,
+// four lose more than 3% against the general form and none more than 8%; what it leaves out of 16 and more
+// entries per row in four and more blocks would gain 2% at most, of shorter rows up to 42%.  Without the slices
+// (pieces below 0.63 of the entries) 65 of 497 lost more than 3%: uniform, 2 per row, 8M rows 277 against 121
+// us, 4 per row, 4M rows 160 / 130.  Taken now: uniform, 16 per row, 4 blocks, 1M rows 101 / 136; R-MAT 22, 8
+// blocks, 254 / 404.
+constexpr double SPM_SLICE = 120.0, SPM_GAIN = 0.70;  // a slice in pieces, an entry's gain in pieces
+static int staged_pays(const tc_part *p, int32_t nb, int32_t W, const DeviceCaps &caps, cudaStream_t s, bool *pays) {
     DevBuf cnt;
     TC_TRY(cnt.alloc(8));
     TC_CUDA(cudaMemsetAsync(cnt.p, 0, 8, s));
@@ -295,7 +300,9 @@ static int staged_pays(const tc_part *p, int32_t W, const DeviceCaps &caps, cuda
     unsigned long long n = 0;
     TC_CUDA(cudaMemcpyAsync(&n, cnt.p, 8, cudaMemcpyDeviceToHost, s));
     TC_CUDA(cudaStreamSynchronize(s));
-    *pays = (double)n - (double)p->R < 0.63 * (double)p->E;
+    const int32_t k = default_merge_range(p->V, caps.sms);
+    const double slices = (double)nb * (double)((p->V + (int64_t)k - 1) / k);
+    *pays = (double)n - (double)p->R + SPM_SLICE * slices < SPM_GAIN * (double)p->E;
     return TC_OK;
 }
 
@@ -308,7 +315,7 @@ static int build_staged(tc_part *p, tc_part *sp, const DeviceCaps &caps, cudaStr
     pp.smem_stage = -1;
     const int32_t nb = (int32_t)(((int64_t)p->V + wmax - 1) / wmax);
     bool pays = false;
-    TC_TRY(staged_pays(p, (p->V + nb - 1) / nb, caps, s, &pays));
+    TC_TRY(staged_pays(p, nb, (p->V + nb - 1) / nb, caps, s, &pays));
     if (!pays) return fail(TC_ERR_UNSUPPORTED, "build_staged: too many pieces");
     TC_TRY(build_partition(p->g, TC_PUSH, nb, &pp, s, sp));
     if (sp->W > wmax || sp->W % 32 != 0 || !sp->id16.p || spm_smem_bytes(sp) > (size_t)caps.max_smem_optin) return fail(TC_ERR_UNSUPPORTED, "build_staged: width");
@@ -507,7 +514,9 @@ extern "C" int tc_spmv_tocab(const tc_part *p, const float *x, float *y, int mem
         TC_CUDA(cudaMemsetAsync(p->sp_err.p, 0, 4, (cudaStream_t)stream));
         TC_TRY(launch_tiled_spmv(sp, p->sp_vals.as<float>(), x, p->sp_err.as<int>(), (cudaStream_t)stream));
         // entries per thread and block: one, two or four, by the mean slice of a block and range (an entry
-        // past them is a round trip of its own)
+        // past them is a round trip of its own, and a place without one costs its slot).  One / two / four, us:
+        // slices of 294 71 / 78 / 84, 383 130 / 143 / 157, 477 267 / 255 / 281, 648 923 / 738 / 838, 941 97 / 97 /
+        // 103, 1,139 194 / 217 / 191, 1,608 299 / 372 / 275
         const int64_t slice = sp->R / ((int64_t)sp->B * sp->nranges);
         auto merge = slice <= SPM_THREADS * 3 / 4   ? k_spmv_merge_staged<4, 1>
                      : slice <= SPM_THREADS * 7 / 4 ? k_spmv_merge_staged<4, 2>

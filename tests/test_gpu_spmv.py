@@ -357,3 +357,32 @@ def test_smem_stage_declines_the_staged_form(T):
     assert torch.equal(declined, general) and size_declined == size
     _, size_staged = product(0)
     assert size_staged > size
+
+
+@pytest.mark.parametrize("V,per_row,B,staged", [(1 << 20, 16, 4, True), (1 << 20, 2, 4, False), (1 << 21, 2, 8, False),
+                                                (150001, 16, 4, True)])
+def test_short_rows_keep_the_general_form(T, V, per_row, B, staged):
+    """The staged form is taken by its pieces, its slices and the entries: not for uniform matrices of few
+    entries per row.  Seen by its memory; the products agree with the sums of small whole numbers exactly."""
+    gen = torch.Generator(device="cuda").manual_seed(2)
+    key = torch.unique(torch.randint(V * V, (per_row * V,), generator=gen, device="cuda"))
+    deg = torch.bincount(key // V, minlength=V)
+    rowptr = torch.cat([deg.new_zeros(1), torch.cumsum(deg, 0)]).to(torch.int32)
+    G = T.graph_load_csr(rowptr, (key % V).to(torch.int32), V=V)
+
+    def used():
+        torch.cuda.synchronize()
+        T.set_device_memory_limit(1 << 50)  # returns the cached blocks
+        T.set_device_memory_limit(0)
+        return T.device_memory_held()
+
+    def product(stage):
+        P = T.tocab_partition(G, T.TC_PUSH, B, smem_stage=stage)
+        before = used()
+        T.part_set_values(P, torch.ones(G.E, device="cuda"))
+        return T.spmv_tocab(P, torch.full((V,), 3.0, device="cuda")), used() - before
+
+    y, size = product(0)
+    general, size_general = product(-1)
+    assert (size > size_general) == staged
+    assert torch.equal(y, 3 * deg.float()) and torch.equal(general, y)
