@@ -315,7 +315,8 @@ typedef struct tc_pr_stats {
  * All blocks read the previous iteration's contributions (Jacobi).  FP32 arithmetic.
  *   ranks_out : [V] floats in params->out_mem space.
  * Errors: TC_ERR_INVALID_ARG (null graph/params/output, damping outside [0,1], iters < 0,
- * partition of another graph or direction), TC_ERR_OOM, TC_ERR_CUDA.
+ * partition of another graph or direction), TC_ERR_OOM, TC_ERR_CUDA, TC_ERR_TIMEOUT (calls with
+ * stats or host output: a bounded device wait gave up).
  */
 int tc_pagerank_pull(const tc_graph *g, const tc_part *part, const tc_pr_params *params,
                      float *ranks_out, tc_pr_stats *stats, void *stream);
@@ -351,8 +352,9 @@ typedef struct tc_bfs_params {
                                  frontier holds fewer than push_threshold * V vertices */
     int32_t resident_edges;   /* push levels only: consecutive levels whose frontier has at most
                                  this many vertices and out-edges run inside ONE launch of a
-                                 thread-block cluster (16 CTAs, else 8), the levels ended by the
-                                 cluster barrier instead of a host round trip (device memory:
+                                 thread-block cluster (16 CTAs, else 8), the levels ended by an
+                                 exchange of the CTAs' counts through distributed shared memory
+                                 instead of a host round trip (device memory:
                                  24 x cluster size x resident_edges bytes, kept with the graph);
                                  the frontier bitmap is rebuilt from the queue before the next
                                  pull level.
@@ -392,7 +394,8 @@ typedef struct tc_bfs_stats {
  * (Sec. 3.3).  With push_threshold > 0, small-frontier levels run top-down from a queue
  * instead (direction optimisation); levels are identical either way.
  * levels_out[v] = hop distance from `source`, -1 when unreachable.
- * Errors: TC_ERR_INVALID_ARG (source outside [0, V)), TC_ERR_OOM, TC_ERR_CUDA.
+ * Errors: TC_ERR_INVALID_ARG (source outside [0, V)), TC_ERR_OOM, TC_ERR_CUDA, TC_ERR_TIMEOUT (the
+ * exchange of a resident level gave up after about a second).
  */
 int tc_bfs_pull(const tc_graph *g, const tc_part *part, int32_t source,
                 const tc_bfs_params *params, int32_t *levels_out, tc_bfs_stats *stats,
@@ -471,8 +474,9 @@ int tc_ppr_set_tuning(tc_graph *g, int32_t hot, int32_t tile);
  * push-pull-push): push over the frontier's out-edges, edge-balanced (compare-and-swap on depth,
  * FP64 atomics on sigma - exact, as every partial sum is an integer below 2^53) while those
  * edges are fewer than 1/14 of the out-edges of the vertices not yet reached (Beamer's rule),
- * else pull over the in-rows of the unreached vertices (a thread per short row, a warp per row
- * of 32 or more in-edges).  Results do not depend on the direction chosen.
+ * else pull over the in-rows of the unreached vertices (one launch: a warp takes 32 vertices, a
+ * lane each for short rows, the whole warp for rows of 32 or more in-edges, and a CTA takes a row
+ * above the graph's hub degree).  Results do not depend on the direction chosen.
  *   out_mem : memory space of depth_out (int32[V]) and sigma_out (double[V]).
  * Synchronises the stream.  Errors: TC_ERR_INVALID_ARG (source outside [0, V), bad out_mem),
  * TC_ERR_OOM, TC_ERR_CUDA.
@@ -490,9 +494,9 @@ int tc_bc_forward(const tc_graph *g, int32_t source, int out_mem, int32_t *depth
  * with both edge directions counts every pair twice).  FP64 throughout, computed as
  * dep[v] = sigma[v] * sum over w of (1 + dep[w]) / sigma[w] (one division per vertex); every
  * product, quotient and sum is rounded separately.  A vertex's out-row is summed by 8 lanes (up
- * to 64 edges), a warp (up to the graph's hub degree, 2048) or a CTA (above it), each lane in
- * strided order and a fixed shuffle or block tree adding the lanes, so the result is
- * deterministic.
+ * to 64 edges), a warp (up to the graph's hub degree, 2048) or a CTA (above it), one launch per
+ * level, each lane in strided order and a fixed shuffle or block tree adding the lanes, so the
+ * result is deterministic.
  *   sources : host int32[num_sources], each in [0, V) (repeats allowed; 0 sources gives zeros).
  *   out_mem : memory space of scores_out (double[V]).
  * Scratch: 3 int32[V] + int64[V] + 3 double[V] (+ double[V] for host output), per call.
@@ -539,7 +543,8 @@ int tc_spmv(const tc_graph *g, const float *vals, const float *x, float *y, int 
  * blocks of x fit one CTA's shared memory (built by the first call; not with smem_stage = -1 or under
  * a memory limit, nor where its memory is not to be had or its pieces would cost more than it gains).
  * The first call takes longer with it and each product less: R-MAT 22 in 8 blocks, 2.9 against
- * 0.7 ms, then 254 against 407 us, so it pays from 15 products on (other matrices 17 to 38); smem_stage = -1 declines it.
+ * 0.7 ms, then 254 against 407 us, so it pays from 15 products on (other matrices 17 to 38);
+ * smem_stage = -1 declines it.
  * For the SpMV of Sec. 4.  Synchronises.
  * Errors: TC_ERR_INVALID_ARG (NULL), TC_ERR_UNSUPPORTED (host values, a renumbered partition),
  * TC_ERR_OOM, TC_ERR_CUDA.

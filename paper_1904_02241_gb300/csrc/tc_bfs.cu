@@ -75,7 +75,7 @@ __device__ __forceinline__ bool scan_warp_rows(unsigned wm, int32_t s, int32_t e
 // The rows of a warp's candidates, a lane each: short rows whole, the first SCAN_PROBE edges of a longer
 // one; the longer rows without a hit there go to the whole warp one after the other, which is what a
 // level waits for (the first pull level of a search on a symmetrised R-MAT 22: 93 us with every long row
-// going there and one edge at a time, 49 us so).
+// going there and one edge at a time, 49 us so).  Probes of 4 to 32 edges: all within 2%.
 constexpr int SCAN_PROBE = 16;
 template <class Bits>
 __device__ __forceinline__ bool scan_rows(bool cand, int32_t s, int32_t e, const int32_t *__restrict__ colidx,
@@ -453,13 +453,14 @@ __global__ void __launch_bounds__(BFS_THREADS) k_bfs_push_edges(const int32_t *_
 // next level has more than `cap` vertices or out-edges.  At the end the claimed vertices are copied,
 // in CTA order, into the host's queue for the next level.  What other CTAs wrote during the launch is
 // read with L2 loads (ld.global.cg), never through L1.
-// Measured on a 2048^2 grid with 5% of its edges removed (some 3,000 levels): 24.6 ms with the frontier kept in
-// global queues and the cluster barrier at every level, 13.0 ms so.
+// Measured on a 2048^2 grid with 5% of its edges removed (some 3,000 levels): 24.2 ms with the frontier kept in
+// global queues and the cluster barrier at every level, 12.7 ms so.
 constexpr int RES_THREADS = 1024;
 constexpr int RES_WARPS = RES_THREADS / 32;
 constexpr int RES_MAX_CTAS = 16;
-constexpr int RES_DEG = 4;      // out-edges of a vertex walked by its own thread
-constexpr int RES_KEEP = 2048;  // claimed vertices per CTA and level whose ranges stay in shared memory
+constexpr int RES_DEG = 4;      // out-edges of a vertex walked by its own thread: 2 / 4 / 8 on that grid 9.8 /
+                                // 10.6 / 10.9 ms back to back
+constexpr int RES_KEEP = 2048;  // claimed vertices per CTA and level whose ranges stay in shared memory (512: the same)
 
 struct ResOut {  // written by CTA 0, thread 0 when the launch ends
     unsigned long long front;  // frontier size of level `lvl`
@@ -1024,7 +1025,10 @@ static int bfs_impl(const tc_graph *cg, const tc_part *part, int32_t source, con
             have_queue = true;
         } else if (use_tocab) {
             // most edges still to scan: the bitmap slice in shared memory, streamed while the frontier is
-            // small (an edge hits with a chance of about m_f / E, so early exit saves little below 1/32)
+            // small (an edge hits with a chance of about m_f / E, so early exit saves little below 1/32).
+            // Two searches on a symmetrised R-MAT of 5M vertices, 8 blocks: a line at 1/2 to 1/64 of the
+            // edges to scan 2,291 to 2,327 us, at all of them (never) 4,158, none (always) 2,505; streaming
+            // below 1/4 to 1/16 of the edges 2,590, 1/32 2,324, 1/64 and 1/128 2,190, always 2,426, never 2,589
             if (blk_grid > 0 && m_u * 4.0 > (double)g->E)
                 k_bfs_block_smem<<<blk_grid, BLK_THREADS, blk_smem, s>>>(
                     part->rowptr.as<int32_t>(), part->colidx.as<int32_t>(), part->id_map.as<int32_t>(), part->R,

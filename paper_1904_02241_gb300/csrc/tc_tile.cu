@@ -11,9 +11,9 @@
 //                padded to a multiple of TILE_WCHUNK;
 //   * heads[]  : one bit per edge, set where a local row starts (uint16 per 16 edges);
 //   * tiles    : every block's rows are cut into row-aligned tiles of about equal estimated
-//                cost (about three waves of CTAs over the device), one CTA each, launched
-//                largest first so that the last wave holds the smallest tiles; every tile of a
-//                block loads the same block values;
+//                cost (one, three or the blocks' own number of waves of CTAs over the device,
+//                see build_tiles), one CTA each, launched largest first so that the last wave
+//                holds the smallest tiles; every tile of a block loads the same block values;
 //   * wtab[]   : per tile, 33 (edge, row) pairs: warp w of the CTA owns the row-aligned edge
 //                range [wtab[w].x, wtab[w+1].x) whose first row is wtab[w].y (equal estimated
 //                cost per warp).
@@ -472,7 +472,9 @@ int build_tiles(tc_part *p, int sms, cudaStream_t s) {
     // equal estimated cost, T = the total over whole waves of one CTA per SM:
     //   * three waves where blocks are uneven (the largest-first order then evens out what the estimate
     //     misses: R-MAT 24 renumbered, 254 us per gather against 278 us with two and 355 us with one);
-    //   * the block count's own waves where the blocks are even (6M uniform: 113 us against 125 us);
+    //   * the block count's own waves where the blocks are even (6M uniform: 113 us against 125 us; 20
+    //     iterations on 3M, 6M, 9M and 12M uniform: 3,573 / 5,222 / 8,453 / 11,295 us against 3,723 / 5,425 /
+    //     8,751 / 11,556 us);
     //   * one wave where a tile costs little next to TILE_SMALL (R-MAT 16: 10 us against 19 us, R-MAT 20
     //     renumbered: 32 us against 35 us).
     DevBuf wrow, cum, cw;
