@@ -160,9 +160,9 @@ class ClockSampler:
 # define the two kernels, the partition and staged format they read, the graph preprocessing
 # before it and the device helpers they use): after any change to those the figure no longer
 # describes the kernels and the bench reports null.
-NCU_TRAFFIC = {("k_tile_gather", 24, 179): 784667392,  # mean of two launches (786.0 and 783.3 MB)
-               ("k_pull_merge_atomic<2>", 24, 179): 349975296}  # (349.8 and 350.1 MB)
-NCU_TRAFFIC_SRC = "b4977289e92a6a36"
+NCU_TRAFFIC = {("k_tile_gather", 24, 179): 784291968,  # mean of two launches (785.7 and 782.8 MB)
+               ("k_pull_merge_atomic<2>", 24, 179): 350063744}  # (349.8 and 350.3 MB)
+NCU_TRAFFIC_SRC = "1529ab7c031eda85"
 
 
 PULL_PATH_SOURCES = ("tc_common_dev.cuh", "tc_graph.cu", "tc_pagerank.cu", "tc_partition.cu", "tc_prims.cu",
@@ -400,7 +400,7 @@ def variants(args, ctx, world):
     lv = torch.empty(gs.V, dtype=torch.int32, device="cuda")
     srcs = gg.sources(gs, args.bfs_sources, seed=13)
     # pure pull (the paper's topology-driven BFS): TOCAB with 8 blocks, every level blocked (the
-    # best of the block and threshold sweeps below), against unblocked; then the same with the
+    # block sweep below has others), against unblocked; then the same with the
     # L2-rule blocks and tau = 0.05, and direction-optimised levels
     P8 = T.tocab_partition(Gs, T.TC_PULL, 8, smem_stage=-1)
     res["bfs_tocab_gteps"] = bfs_rate(T, Gs, P8, srcs, lv, stream, 0.0, 0.0)[0]

@@ -258,8 +258,10 @@ def pagerank_push(graph: Graph, part: Partition | None = None, damping: float = 
                   profile: bool = False, stream=None, return_stats: bool = False, lb_warp_min: int = 0,
                   sums: str = "fixed"):
     """tc_pagerank_push (Alg. 2; TOCAB Alg. 5 when part is given).  sums="fixed": 64-bit
-    fixed-point reductions (bitwise repeatable); "float": FP32 atomics.  lb_warp_min = 0: a
-    thread per edge; > 0: the thread/warp/CTA row mapping with that warp threshold."""
+    fixed-point reductions (bitwise repeatable); "float": FP32 atomics.  lb_warp_min = 0: by
+    destination ranges with part and fixed sums (built by the call that brings the iterations asked
+    of part to three), else a thread per edge; > 0: the thread/warp/CTA row mapping with that warp
+    threshold."""
     r, st = _pagerank(L.load().tc_pagerank_push, "tc_pagerank_push", graph, part, damping, iters, dangling, out,
                       init, profile, stream, sums, lb_warp_min)
     return (r, st) if return_stats else r
@@ -310,7 +312,8 @@ def spmv(matrix: Graph, vals: torch.Tensor, x: torch.Tensor, out: torch.Tensor |
 
 def part_set_values(part: "Partition", vals: torch.Tensor, stream=None):
     """tc_part_set_values: the matrix values (CSR order, float32 on the device) for SpMV with
-    TOCAB: GC-pull on a TC_PUSH partition, GC-push on a TC_PULL one."""
+    TOCAB: GC-pull on a TC_PUSH partition (large ones staged: a longer first call, shorter products;
+    smem_stage=-1 declines it), GC-push on a TC_PULL one."""
     if vals.dtype != torch.float32 or not vals.is_cuda or not vals.is_contiguous():
         raise ValueError("vals must be a contiguous float32 CUDA tensor")
     _check(L.load().tc_part_set_values(part.handle, vals.data_ptr() if vals.numel() else None, L.TC_MEM_DEVICE,
