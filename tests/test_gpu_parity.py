@@ -2,6 +2,8 @@
 
 Integer work (transpose, partition, BFS levels) must match bit-exactly; FP32 PageRank
 must be within an L1 relative error of 1e-5 of the FP64 oracle after 20 iterations."""
+import gc
+
 import numpy as np
 import pytest
 import torch
@@ -987,6 +989,7 @@ def test_push_builds_its_destination_ranges_when_they_pay(T):
     G = _load(T, g)
 
     def used():
+        gc.collect()  # handles of earlier tests
         torch.cuda.synchronize()
         T.set_device_memory_limit(1 << 50)  # returns the cached blocks
         T.set_device_memory_limit(0)

@@ -4,6 +4,7 @@ lane, then a 5-level shuffle tree), so row i may differ from the exact product b
 summation whose longest chain has at most d_i + 5 roundings.  The inputs are the same FP32 values
 on both sides."""
 import ctypes as C
+import gc
 import subprocess
 
 import numpy as np
@@ -337,6 +338,7 @@ def test_smem_stage_declines_the_staged_form(T):
     x = torch.from_numpy(rng.standard_normal(V).astype(np.float32)).cuda()
 
     def used():
+        gc.collect()  # handles of earlier tests
         torch.cuda.synchronize()
         T.set_device_memory_limit(1 << 50)  # returns the cached blocks
         T.set_device_memory_limit(0)
@@ -371,6 +373,7 @@ def test_short_rows_keep_the_general_form(T, V, per_row, B, staged):
     G = T.graph_load_csr(rowptr, (key % V).to(torch.int32), V=V)
 
     def used():
+        gc.collect()  # handles of earlier tests
         torch.cuda.synchronize()
         T.set_device_memory_limit(1 << 50)  # returns the cached blocks
         T.set_device_memory_limit(0)
